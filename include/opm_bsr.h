@@ -98,7 +98,12 @@ enum {
 /* Launch structure of the sweeps over the schedule's phases (runs of
  * mutually independent rows: the levels or colours). */
 enum {
-  OPM_SWEEP_AUTO = 0,        /* per-phase launches up to 1024 phases        */
+  OPM_SWEEP_AUTO = 0,        /* a single system of up to about 300,000 rows:
+                                one cooperative launch that refactors and
+                                solves it, with bounded grid barriers between
+                                its stages; otherwise per-phase launches up
+                                to 1024 phases, cooperative sweeps past that.
+                                Every form gives the same bits              */
   OPM_SWEEP_PER_PHASE = 1,   /* one kernel launch per phase                 */
   OPM_SWEEP_COOPERATIVE = 2  /* one cooperative launch walking all phases,
                                 with a bounded grid barrier between them    */
@@ -115,7 +120,7 @@ typedef struct opm_options {
                             0 = default (2,000,000)                           */
   int32_t debug_skip_item; /* test hook, -1 = off: the CTA with this index
                             never arrives at the grid barriers of the
-                            cooperative sweep kernels, so the other CTAs'
+                            cooperative launches, so the other CTAs'
                             waits expire after spin_limit_us
                             (OPM_ERR_TIMEOUT)                                */
   int32_t profile_kernels; /* nonzero: record CUDA events around every kernel

@@ -111,6 +111,7 @@ opm_status tune(Problem &P, bool allow_natural, int32_t repeats, const opm_optio
   if (allow_natural) scheds.push_back(OPM_SCHED_NATURAL);
   for (int32_t sc : scheds) {
     const int32_t phases = tryc({sc, OPM_SWEEP_COOPERATIVE, 2, 0});
+    tryc({sc, OPM_SWEEP_AUTO, 2, 0});
     if (phases <= 1024) tryc({sc, OPM_SWEEP_PER_PHASE, 2, 0});
   }
   // 2. iterations per loop body
@@ -119,7 +120,7 @@ opm_status tune(Problem &P, bool allow_natural, int32_t repeats, const opm_optio
     for (int32_t ch : {1, 4}) tryc({b.schedule, b.sweep_launch, ch, b.small_phase_slices});
   }
   // 3. small-phase threshold of the per-phase launches
-  if (rep.best >= 0 && rep.cand[rep.best].sweep_launch == OPM_SWEEP_PER_PHASE) {
+  if (rep.best >= 0 && rep.cand[rep.best].sweep_launch != OPM_SWEEP_COOPERATIVE) {
     const opm_tune_entry b = rep.cand[rep.best];
     for (int32_t sm : {-1, 1 << 30}) tryc({b.schedule, b.sweep_launch, b.chunk, sm});
   }

@@ -149,6 +149,80 @@ __device__ __forceinline__ void one_pass_rows(const Sys &S, int sl, bool fz, con
   }
 }
 
+// Eliminates the lane's row with its pivots k < i (Algorithm 2's updates of
+// row i), its blocks being in their factor slots.  All lanes of the warp call
+// it; lanes with !gen only take part in the walk.
+template <typename TF>
+__device__ __forceinline__ void eliminate_row(const Sys &S, int sl, bool gen, TF *lu) {
+  const int lane = threadIdx.x & 31;
+  const int s0 = sl * 32;
+  const int i = s0 + lane;
+  const int n = S.n;
+  const unsigned lt = lanemask_lt();
+  const int lrow = (i < n) ? __ldg(S.l_rp + i) : 0;
+  const int len = (i < n) ? __ldg(S.l_rp + i + 1) - lrow : 0;
+  int base = (s0 < n) ? __ldg(S.l_rp + s0) : 0;
+  const int maxlen = __reduce_max_sync(0xffffffffu, gen ? len : 0);
+  for (int k = 0; k < maxlen; ++k) {
+    const unsigned m = __ballot_sync(0xffffffffu, len > k);
+    if (gen && len > k) {
+      const int cnt = __popc(m);
+      const int q = __popc(m & lt);
+      const int kc = __ldg(S.l_col + base + q);
+      TF *Lp = lu + 9ll * base + q;
+      const TF *Dk = lu + S.d_off + (int64_t)kSliceVals * (kc >> 5) + (kc & 31);
+      TF a[9], d[9], l[9];
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        a[c] = Lp[c * cnt];
+        d[c] = __ldcg(Dk + 32 * c);
+      }
+      // L_ik = A_ik * inv(U_kk)
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+          l[3 * r + c] = fma(a[3 * r], d[c], fma(a[3 * r + 1], d[3 + c], a[3 * r + 2] * d[6 + c]));
+#pragma unroll
+      for (int c = 0; c < 9; ++c) Lp[c * cnt] = l[c];
+      // A_ij -= L_ik * U_kj for the listed j
+      const int u1 = __ldg(S.upd_ptr + lrow + k + 1);
+      for (int u = __ldg(S.upd_ptr + lrow + k); u < u1; ++u) {
+        const int64_t ds = __ldg(S.upd_dst + u), ss = __ldg(S.upd_src + u);
+        TF *Ap = lu + (ds >> 6);
+        const int dstr = (int)(ds & 63);
+        const TF *Up = lu + (ss >> 6);
+        const int sstr = (int)(ss & 63);
+        TF uu[9];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) uu[c] = __ldcg(Up + c * sstr);
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            TF *ap = Ap + (3 * r + c) * dstr;
+            *ap = fma(-l[3 * r], uu[c], fma(-l[3 * r + 1], uu[3 + c], fma(-l[3 * r + 2], uu[6 + c], *ap)));
+          }
+      }
+    }
+    base += __popc(m);
+  }
+}
+
+// Inverts the row's diagonal block, held in D (in_regs) or in its slot, into
+// the slot; false for a singular block.
+template <typename TF>
+__device__ __forceinline__ bool invert_diagonal(const Sys &S, int sl, bool in_regs, const TF (&D)[9], TF *lu) {
+  TF *Dp = lu + S.d_off + (int64_t)kSliceVals * sl + (threadIdx.x & 31);
+  TF a[9], o[9];
+#pragma unroll
+  for (int c = 0; c < 9; ++c) a[c] = in_regs ? D[c] : Dp[32 * c];
+  const bool ok = inv3<TF>(a, o);
+#pragma unroll
+  for (int c = 0; c < 9; ++c) Dp[32 * c] = o[c];
+  return ok;
+}
+
 // ILU0 decomposition (Algorithm 2) of the permuted matrix, phase by phase,
 // fused with the value permutation: with vals_in, block w of the permuted
 // matrix is copied from the caller's block a_src[w] (Algorithm 3's index
@@ -163,87 +237,30 @@ __device__ __forceinline__ void one_pass_rows(const Sys &S, int sl, bool fz, con
 // copy reads only the caller's values and writes only the phase's own rows,
 // so it overlaps the tail of the previous phase; the elimination, which
 // reads earlier phases' pivots, comes after the wait.
+// Returns false for a lane whose row has a singular pivot.
 template <typename TF, bool ONE_PASS, bool EARLY_COPY = false, bool DREG = true>
-__device__ __forceinline__ void factor_rows(const Sys &S, int sl, int r0, int r1) {
-  if (S.skip) return;  // warp-uniform: the entry belongs to one system
+__device__ __forceinline__ bool factor_rows(const Sys &S, int sl, int r0, int r1) {
   const int lane = threadIdx.x & 31;
-  const int s0 = sl * 32;
-  const int i = s0 + lane;
-  const int n = S.n;
+  const int i = sl * 32 + lane;
   const bool act = i >= r0 && i < r1;
   const bool fz = ONE_PASS && act && ((__ldg(S.fz_mask + sl) >> lane) & 1u);
   const bool gen = act && !fz;
   TF *lu = static_cast<TF *>(S.lu);
   const double *__restrict__ vals_user = S.vals_in;
-  const unsigned lt = lanemask_lt();
-  DevState *st = S.st;
   TF D[9];
   if (ONE_PASS && __any_sync(0xffffffffu, fz)) one_pass_rows<TF, DREG>(S, sl, fz, vals_user, lu, D);
   if (__any_sync(0xffffffffu, gen)) {
     copy_row_to_factors<TF>(S, sl, gen, vals_user, lu);
     if (EARLY_COPY) pdl_wait();
-    // ---- eliminate with the pivots k < i (Algorithm 2's updates of row i)
-    const int lrow = (i < n) ? __ldg(S.l_rp + i) : 0;
-    const int len = (i < n) ? __ldg(S.l_rp + i + 1) - lrow : 0;
-    int base = (s0 < n) ? __ldg(S.l_rp + s0) : 0;
-    const int maxlen = __reduce_max_sync(0xffffffffu, gen ? len : 0);
-    for (int k = 0; k < maxlen; ++k) {
-      const unsigned m = __ballot_sync(0xffffffffu, len > k);
-      if (gen && len > k) {
-        const int cnt = __popc(m);
-        const int q = __popc(m & lt);
-        const int kc = __ldg(S.l_col + base + q);
-        TF *Lp = lu + 9ll * base + q;
-        const TF *Dk = lu + S.d_off + (int64_t)kSliceVals * (kc >> 5) + (kc & 31);
-        TF a[9], d[9], l[9];
-#pragma unroll
-        for (int c = 0; c < 9; ++c) {
-          a[c] = Lp[c * cnt];
-          d[c] = __ldcg(Dk + 32 * c);
-        }
-        // L_ik = A_ik * inv(U_kk)
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            l[3 * r + c] = fma(a[3 * r], d[c], fma(a[3 * r + 1], d[3 + c], a[3 * r + 2] * d[6 + c]));
-#pragma unroll
-        for (int c = 0; c < 9; ++c) Lp[c * cnt] = l[c];
-        // A_ij -= L_ik * U_kj for the listed j
-        const int u1 = __ldg(S.upd_ptr + lrow + k + 1);
-        for (int u = __ldg(S.upd_ptr + lrow + k); u < u1; ++u) {
-          const int64_t ds = __ldg(S.upd_dst + u), ss = __ldg(S.upd_src + u);
-          TF *Ap = lu + (ds >> 6);
-          const int dstr = (int)(ds & 63);
-          const TF *Up = lu + (ss >> 6);
-          const int sstr = (int)(ss & 63);
-          TF uu[9];
-#pragma unroll
-          for (int c = 0; c < 9; ++c) uu[c] = __ldcg(Up + c * sstr);
-#pragma unroll
-          for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              TF *ap = Ap + (3 * r + c) * dstr;
-              *ap = fma(-l[3 * r], uu[c], fma(-l[3 * r + 1], uu[3 + c], fma(-l[3 * r + 2], uu[6 + c], *ap)));
-            }
-        }
-      }
-      base += __popc(m);
-    }
+    eliminate_row<TF>(S, sl, gen, lu);
   }
-  if (act) {
-    TF *Dp = lu + S.d_off + (int64_t)kSliceVals * sl + lane;
-    TF a[9], o[9];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) a[c] = (fz && DREG) ? D[c] : Dp[32 * c];
-    if (!inv3<TF>(a, o)) {
-      atomicCAS(&st->error, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
-      atomicMin(&st->err_row, i);
-    }
-#pragma unroll
-    for (int c = 0; c < 9; ++c) Dp[32 * c] = o[c];
-  }
+  return !act || invert_diagonal<TF>(S, sl, fz && DREG, D, lu);
+}
+
+// Records a singular pivot of the lane's row for the host.
+__device__ __forceinline__ void record_singular(DevState *st, int i) {
+  atomicCAS(&st->error, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
+  atomicMin(&st->err_row, i);
 }
 
 // One launch per phase, one 32-row slice per warp.  ONE_PASS takes the
@@ -268,7 +285,10 @@ __global__ void __launch_bounds__(256, MINB) k_factor_phase(Batch B, int c) {
   const int e = __ldg(B.fwd_ptr + c) + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (e >= __ldg(B.fwd_ptr + c + 1)) return;
   const int4 E = B.ent[e];
-  factor_rows<TF, ONE_PASS, !ONE_PASS, DREG>(B.sys[E.x], E.y, E.z, E.w);
+  const Sys &S = B.sys[E.x];
+  if (S.skip) return;  // warp-uniform: the entry belongs to one system
+  if (!factor_rows<TF, ONE_PASS, !ONE_PASS, DREG>(S, E.y, E.z, E.w))
+    record_singular(S.st, E.y * 32 + (threadIdx.x & 31));
 }
 
 template <typename TF>
@@ -281,7 +301,9 @@ __global__ void __launch_bounds__(1024) k_factor(Batch B) {
     const int e1 = __ldg(B.fwd_ptr + c + 1);
     for (int e = __ldg(B.fwd_ptr + c) + g; e < e1; e += W) {
       const int4 E = B.ent[e];
-      factor_rows<TF, false>(B.sys[E.x], E.y, E.z, E.w);
+      const Sys &S = B.sys[E.x];
+      if (!S.skip && !factor_rows<TF, false>(S, E.y, E.z, E.w))
+        record_singular(S.st, E.y * 32 + (threadIdx.x & 31));
     }
   }
 }

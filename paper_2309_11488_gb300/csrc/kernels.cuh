@@ -21,9 +21,9 @@
 // 4.4).  The sweeps walk the phases in order, either one launch per phase
 // or one cooperative launch with a bounded grid barrier between phases.
 //
-// Reductions: per system in a fixed order (see red_end and
-// last_cta_reduce); the warp or CTA that completes a system's sum runs the
-// scalar part of BiCGStab (alpha, omega, beta, the stopping rule).
+// Reductions: per system in a fixed order (see red_end); the warp that
+// completes a system's sum runs the scalar part of BiCGStab (alpha, omega,
+// beta, the stopping rule).
 #pragma once
 
 #include <cstdint>
@@ -35,10 +35,10 @@ namespace opm {
 enum SweepMode { kModePlain = 0, kModeP = 1, kModeS = 2 };
 
 // One system's device data.  The last group of fields is set per call.
-struct Sys {
+struct alignas(16) Sys {
   int32_t n, nslices, ntiles, nphases;
   int32_t ntiles_s;  // 256-row tiles of the SpMV kernels
-  int32_t pad0;
+  int32_t tree;      // order of the sums within a tile (see red_end)
   const int32_t *perm;
   const int32_t *a_rp, *a_col, *a_src;
   const int64_t *a_dst;
@@ -182,7 +182,10 @@ __device__ __forceinline__ bool inv3(const T (&a)[9], T (&o)[9]) {
 //
 // A per-system sum of NV values without CTA-wide barriers, in a fixed order:
 // every warp sums its lanes (xor butterfly); the last warp of the CTA to
-// finish adds the CTA's warp sums in warp order (the tile's partial); the
+// finish adds the CTA's eight warp sums (the tile's partial: the butterfly
+// for systems of the resident kernel's sizes, whose unit sums it reduces the
+// same way; in warp order with S.tree, for larger ones and for the iterative
+// sweeps); the
 // last tile of each group of 32 tiles adds the group's tile partials (xor
 // butterfly over 32 lanes); the last group of the system adds the group
 // partials (strided over the lanes, then the butterfly).  Warps that are not
@@ -207,6 +210,46 @@ __device__ __forceinline__ void warp_sum(double (&v)[NV]) {
   }
 }
 
+// The warp sums of NV <= 3 values with fewer additions than NV butterflies: a
+// halving exchange leaves each half (quarter) of the lanes with one value,
+// whose own butterfly goes on from there.  The same pairs are added in the
+// same order as in warp_sum, so the bits are the same; 5, 6 additions per
+// lane for two, three values instead of 10, 15 (an FP64 addition costs as
+// much as an FMA of the row work, and the pipe bounds these kernels).
+// Returns value warp_sum_of(lane)'s sum, -1 marking lanes that hold a copy.
+template <int NV>
+__device__ __forceinline__ double warp_sum_split(const double (&v)[NV]) {
+  static_assert(NV >= 1 && NV <= 3, "one to three values");
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool hi = lane & 16;
+  double t;
+  if constexpr (NV == 1) {
+    t = v[0] + __shfl_xor_sync(all, v[0], 16);
+    t += __shfl_xor_sync(all, t, 8);
+  } else if constexpr (NV == 2) {
+    t = (hi ? v[1] : v[0]) + __shfl_xor_sync(all, hi ? v[0] : v[1], 16);
+    t += __shfl_xor_sync(all, t, 8);
+  } else {
+    // lanes < 16 keep values 0 and 1, the others value 2
+    const double u0 = (hi ? v[2] : v[0]) + __shfl_xor_sync(all, hi ? v[0] : v[2], 16);
+    const double u1 = v[1] + __shfl_xor_sync(all, v[1], 16);
+    const bool one = !hi && (lane & 8);
+    t = (one ? u1 : u0) + __shfl_xor_sync(all, (hi || (lane & 8)) ? u0 : u1, 8);
+  }
+  t += __shfl_xor_sync(all, t, 4);
+  t += __shfl_xor_sync(all, t, 2);
+  t += __shfl_xor_sync(all, t, 1);
+  return t;
+}
+
+template <int NV>
+__device__ __forceinline__ int warp_sum_of(int lane) {
+  if constexpr (NV == 1) return lane == 0 ? 0 : -1;
+  else if constexpr (NV == 2) return (lane & 15) == 0 ? lane >> 4 : -1;
+  else return lane == 0 ? 0 : lane == 8 ? 1 : lane == 16 ? 2 : -1;
+}
+
 // Called by every thread at kernel start (one CTA barrier).
 template <int NV>
 __device__ __forceinline__ void red_begin(RedShared<NV> &rs) {
@@ -221,16 +264,24 @@ template <int NV>
 __device__ __noinline__ bool red_tail(RedShared<NV> &rs, const Sys &S, int tile, int ntiles, int nw, int lane,
                                       double (&tot)[NV]) {
   unsigned t = 0;
-  // the tile's partial, warps in order
+  // the tile's partial from its warps' sums
   const int g = tile >> 5, ng = (ntiles + 31) >> 5, gsize = min(32, ntiles - 32 * g);
+  double p[NV];
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    if (S.tree) {
+      p[q] = 0.0;
+#pragma unroll 1
+      for (int ww = 0; ww < nw; ++ww) p[q] += rs.wsum[ww][q];
+    } else {
+      p[q] = lane < nw ? rs.wsum[lane][q] : 0.0;
+#pragma unroll
+      for (int o = kMaxWarps / 2; o > 0; o >>= 1) p[q] += __shfl_xor_sync(0xffffffffu, p[q], o);
+    }
+  }
   if (lane == 0) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      double p = 0.0;
-#pragma unroll 1
-      for (int ww = 0; ww < nw; ++ww) p += rs.wsum[ww][q];
-      S.partials[(size_t)tile * NV + q] = p;
-    }
+    for (int q = 0; q < NV; ++q) S.partials[(size_t)tile * NV + q] = p[q];
     __threadfence();
     t = atomicAdd(&S.grp_count[g], 1u);
   }
@@ -272,11 +323,12 @@ template <int NV>
 __device__ __forceinline__ bool red_end(double (&v)[NV], RedShared<NV> &rs, const Sys &S, int tile, int ntiles,
                                         double (&tot)[NV]) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  warp_sum<NV>(v);
+  const double sum = warp_sum_split<NV>(v);
+  const int q = warp_sum_of<NV>(lane);
+  if (q >= 0) rs.wsum[w][q] = sum;
+  __syncwarp();
   unsigned t = 0;
   if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) rs.wsum[w][q] = v[q];
     __threadfence_block();
     t = atomicAdd(&rs.count, 1u);
   }
@@ -288,10 +340,12 @@ __device__ __forceinline__ bool red_end(double (&v)[NV], RedShared<NV> &rs, cons
 
 // The second form: a CTA-wide tree in shared memory (values leave the
 // registers at once), then the system's last CTA sums the tile partials in
-// tile order.  k_spmv_t's three sums use it: measured on GB300 its launch
-// takes 147 us this way against 172 us with red_end (same arithmetic order
-// class, both deterministic), while the one- and two-value kernels are
-// faster with red_end (k_spmv_v 135 against 140 us).
+// tile order.  k_spmv_t's three sums use it for systems past the resident
+// kernel's sizes (S.tree): at the 949,871-cell system its launch takes 3 us
+// less than with red_end with the product reuse, 10 us less without (an
+// addition per warp costs the FP64 pipe as much as an FMA, and the tree has
+// fewer), while the one- and two-value kernels are faster with red_end
+// (k_spmv_v 135 against 140 us).
 constexpr int kRedThreads = 256;
 
 template <int NV>
@@ -643,14 +697,19 @@ __global__ void __launch_bounds__(256, 8) k_spmv_v(Batch B) {
   }
 }
 
+// Whether none, all or some of a launch's systems have their sums in the
+// tree's order (Sys::tree).
+enum TreeMode { kTreeNone = 0, kTreeAll = 1, kTreeMixed = 2 };
+
 // t = A s^, (t,s), (t,t), (s,s); the half-step test and omega.  REUSE as
 // for k_spmv_v.  WIDE: eight CTAs per SM (32 registers; with REUSE its
 // three sums spill 56 bytes per thread), for launches with more tiles than
 // six CTAs per SM hold; otherwise (REUSE) six CTAs per SM and no spill,
 // which a small system's latency-bound product prefers.
-template <bool REUSE, bool WIDE = true>
+template <bool REUSE, bool WIDE, int TREE>
 __global__ void __launch_bounds__(256, (REUSE && !WIDE) ? 6 : 8) k_spmv_t(Batch B) {
-
+  __shared__ RedShared<3> rs_;
+  if (TREE != kTreeAll) red_begin<3>(rs_);
   pdl_enter();
   OPM_TILE_S(B, S, lt);
   if (!running(S.st)) return;
@@ -670,7 +729,9 @@ __global__ void __launch_bounds__(256, (REUSE && !WIDE) ? 6 : 8) k_spmv_t(Batch 
     }
   }
   double tot[3];
-  if (last_cta_reduce<3>(acc, S, lt, S.ntiles_s, tot) && threadIdx.x == 0) {
+  const bool tree = TREE == kTreeAll || (TREE == kTreeMixed && S.tree);
+  if (tree ? last_cta_reduce<3>(acc, S, lt, S.ntiles_s, tot) && threadIdx.x == 0
+           : red_end<3>(acc, rs_, S, lt, S.ntiles_s, tot) && (threadIdx.x & 31) == 0) {
     DevState *st = S.st;
     st->ts = tot[0];
     st->tt = tot[1];

@@ -3,7 +3,9 @@
 // A handle owns one system's schedule-ordered device copy of the matrix, its
 // ILU0 factors and its Krylov vectors.  Work is launched through a Runner: a
 // set of systems (a handle's own set of one, or a batch of handles) with its
-// work lists, its kernel-parameter block and three CUDA graphs:
+// work lists and its kernel-parameter block.  A single system of the resident
+// kernel's sizes (resident_size) is refactored and solved by one launch of
+// it; everything else goes through three CUDA graphs:
 //   * factor graph: clear errors -> ILU0 phases -> record errors -> results;
 //   * solve graph: setup -> while (any system running) { `chunk` BiCGStab
 //     iterations; loop condition } -> true residual -> results.  The loop
@@ -27,6 +29,7 @@
 #include "factor.cuh"
 #include "gmres.cuh"
 #include "iterative.cuh"
+#include "resident.cuh"
 
 using namespace opm;
 
@@ -102,6 +105,11 @@ struct Runner {
   cudaGraphExec_t solve_exec = nullptr, iter_exec = nullptr, factor_exec = nullptr;
   cudaGraphExec_t fs_exec = nullptr;  // refactor + solve in one graph (setup beside the factorisation)
   int iter_launches = 0, factor_launches = 0;
+  int tree = kTreeNone;   // which systems' sums take the tree's order (Sys::tree)
+  bool resident = false;  // factorisation and solve run in the resident kernel
+  Resident RA{};          // its arguments
+  const void *res_kernel = nullptr;
+  int res_grid = 1, res_threads = 256;
   std::vector<cudaEvent_t> kev;  // profiling events, 6 per iteration of a chunk
   cudaEvent_t ev_done = nullptr;
 };
@@ -405,6 +413,13 @@ int launch_factor_seq(Runner &R, cudaStream_t st) {
   return n + 2;
 }
 
+template <int TREE>
+void launch_spmv_t(Runner &R, cudaStream_t st) {
+  if (R.reuse && R.ntiles_s > 6 * R.sms) launch_pdl(k_spmv_t<true, true, TREE>, R.ntiles_s, 256, st, R.B);
+  else if (R.reuse) launch_pdl(k_spmv_t<true, false, TREE>, R.ntiles_s, 256, st, R.B);
+  else launch_pdl(k_spmv_t<false, true, TREE>, R.ntiles_s, 256, st, R.B);
+}
+
 // One BiCGStab iteration.  With ev (6 events), the kernel groups are
 // bracketed by event-record nodes (external records, so that they become
 // real graph nodes) for per-kernel timing.
@@ -429,9 +444,9 @@ int launch_iteration(Runner &R, cudaStream_t st, cudaEvent_t *ev) {
     launch_pdl(k_wells, R.nsys, 256, st, R.B, 1);
     ++n;
   }
-  if (R.reuse && R.ntiles_s > 6 * R.sms) launch_pdl(k_spmv_t<true, true>, R.ntiles_s, 256, st, R.B);
-  else if (R.reuse) launch_pdl(k_spmv_t<true, false>, R.ntiles_s, 256, st, R.B);
-  else launch_pdl(k_spmv_t<false>, R.ntiles_s, 256, st, R.B);
+  if (R.tree == kTreeNone) launch_spmv_t<kTreeNone>(R, st);
+  else if (R.tree == kTreeAll) launch_spmv_t<kTreeAll>(R, st);
+  else launch_spmv_t<kTreeMixed>(R, st);
   mark(4);
   launch_pdl(k_update, R.ntiles, 256, st, R.B);
   mark(5);
@@ -605,6 +620,22 @@ void runner_destroy(Runner *R) {
   delete R;
 }
 
+// Sizes of the resident kernel, in 32-row slices of a system.  A trio per
+// slice up to 2.5 slices per trio, 60,800 rows on 152 SMs, then a warp per
+// slice up to two slices per warp, 311,296 rows; past that the launches per
+// phase.  Measured, refactor + solve at rtol 1e-3 in us (launches per phase,
+// trios, warps): 3,868 rows 553, 337, 570; 31,105 rows 726, 513, 727; 60,793
+// rows 912, 776, 786; 105,006 rows 1268, 1104, 907; 249,053 rows 1676, 2042,
+// 1309; 354,590 rows 1824, 2707, 1862; 949,871 rows 3482, 6449, 3729.
+bool resident_trios(int nslices, int sms) { return 2 * (int64_t)nslices <= 5 * (int64_t)kTrios * sms; }
+bool resident_size(int nslices, int sms) { return nslices <= 2 * (kResidentThreads / 32) * (int64_t)sms; }
+
+// A system's order of summation follows from its size and the sweeps alone,
+// so it is the same in every launch form, alone and in a batch.
+int32_t tree_order(const Runner &R, const opm_solver *h) {
+  return R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(h->nslices, R.sms);
+}
+
 // Work lists and graphs for a set of analysed, allocated systems.
 // Whether the BiCGStab products after an application take their upper sums
 // from the backward sweep (Sys::uz): FP64 factors (an FP32 U is not A's to
@@ -619,6 +650,116 @@ uint64_t spin_ns(const opm_options &o) {
 }
 
 int chunk_of(const opm_options &o) { return o.chunk > 0 ? o.chunk : 2; }
+
+template <typename TF>
+const void *resident_kernel(bool trio) {
+  return trio ? (const void *)k_resident<TF, true, kTrioThreads> : (const void *)k_resident<TF, false, kResidentThreads>;
+}
+
+// Whether the runner's system goes to the resident kernel, and its work lists.
+opm_status resident_create(Runner &R, int max_entries) {
+  if (R.nsys > 1 || R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(R.nall, R.sms)) return OPM_OK;
+  const bool trio = resident_trios(R.nall, R.sms);
+  R.res_kernel = R.fp32 ? resident_kernel<float>(trio) : resident_kernel<double>(trio);
+  R.res_threads = trio ? kTrioThreads : kResidentThreads;
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, R.res_kernel, R.res_threads, sizeof(ResShared)) !=
+          cudaSuccess ||
+      occ < 1) {
+    cudaGetLastError();
+    return OPM_OK;
+  }
+  R.res_grid = std::max(1, std::min(R.sms * occ, std::max(max_entries, R.nall)));
+  std::vector<int32_t> off_s(1, 0), off_u(1, 0), goff_s(1, 0), goff_u(1, 0);
+  std::vector<int2> grp_s, grp_u;
+  for (int s = 0; s < R.nsys; ++s) {
+    const Sys &S = R.mem[s]->sys;
+    off_s.push_back(off_s.back() + 8 * S.ntiles_s);
+    off_u.push_back(off_u.back() + 8 * S.ntiles);
+    for (int g = 0; g < (S.ntiles_s + 31) / 32; ++g) grp_s.push_back(make_int2(s, g));
+    for (int g = 0; g < (S.ntiles + 31) / 32; ++g) grp_u.push_back(make_int2(s, g));
+    goff_s.push_back((int32_t)grp_s.size());
+    goff_u.push_back((int32_t)grp_u.size());
+  }
+  // units of the products, heaviest 256-row tiles first: dealt round robin
+  // over the warps, the last round is then the cheapest
+  std::vector<int4> prod;
+  std::vector<int64_t> work;
+  for (int s = 0; s < R.nsys; ++s) {
+    const Analysis &an = R.mem[s]->an;
+    for (int sl = 0; sl < R.mem[s]->nslices; ++sl) {
+      const int t = sl / 8, r0 = t * kSpmvRows, r1 = std::min(an.n, r0 + kSpmvRows);
+      prod.push_back(make_int4(s, sl, 0, an.n));
+      work.push_back(R.reuse && t < (int)an.sp_tile.size() ? an.sp_tile[t] : an.a_rowptr[r1] - an.a_rowptr[r0]);
+    }
+  }
+  {
+    std::vector<int> ord(prod.size());
+    for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int)q;
+    std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return work[a] > work[b]; });
+    std::vector<int4> sorted(prod.size());
+    for (size_t q = 0; q < ord.size(); ++q) sorted[q] = prod[ord[q]];
+    prod.swap(sorted);
+  }
+  Resident &A = R.RA;
+  int4 *d_prod;
+  if (opm_status sp = upload(R.allocs, R.dev_bytes, R.stream, &d_prod, prod); sp != OPM_OK) return sp;
+  A.prod = d_prod;
+  int32_t *d_os, *d_ou, *d_gos, *d_gou;
+  int2 *d_gs, *d_gu;
+  opm_status s;
+  if ((s = upload(R.allocs, R.dev_bytes, R.stream, &d_os, off_s)) != OPM_OK ||
+      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_ou, off_u)) != OPM_OK ||
+      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gos, goff_s)) != OPM_OK ||
+      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gou, goff_u)) != OPM_OK ||
+      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gs, grp_s)) != OPM_OK ||
+      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gu, grp_u)) != OPM_OK)
+    return s;
+  const size_t ns = (size_t)off_s.back(), nu = (size_t)off_u.back();
+  double *sum_s, *sum_u;
+  if ((s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_s, 3 * ns)) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_u, 3 * nu)) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.gpart, 3 * std::max(grp_s.size(), grp_u.size()))) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.err, 2 * (size_t)R.nsys)) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.ctl, 1)) != OPM_OK)
+    return s;
+  // the last tile of a system may have fewer than eight slices: the units
+  // past them stay zero
+  CK(cudaMemsetAsync(sum_s, 0, sizeof(double) * 3 * ns, R.stream));
+  CK(cudaMemsetAsync(sum_u, 0, sizeof(double) * 3 * nu, R.stream));
+  CK(cudaMemsetAsync(A.err, 0, sizeof(int32_t) * 2 * R.nsys, R.stream));
+  CK(cudaMemsetAsync(A.ctl, 0, sizeof(ResidentCtl), R.stream));
+  A.B = R.B;
+  A.ds = {sum_s, d_os, d_gs, d_gos, (int)grp_s.size(), off_s.back()};
+  A.du = {sum_u, d_ou, d_gu, d_gou, (int)grp_u.size(), off_u.back()};
+  A.nupd = 8 * R.ntiles;
+  A.res = R.h_res;
+  R.resident = true;
+  return OPM_OK;
+}
+
+// Enqueues the resident kernel.
+opm_status resident_enqueue(Runner &R, bool factor, bool solve) {
+  if (R.nsys == 1) {
+    R.RA.one = R.mem[0]->sys;
+    if (!R.reuse) R.RA.one.uz = nullptr;
+  }
+  R.RA.work = (factor ? kResFactor : 0) | (solve ? kResSolve : 0);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)R.res_grid);
+  cfg.blockDim = dim3((unsigned)R.res_threads);
+  cfg.dynamicSmemBytes = sizeof(ResShared);
+  cfg.stream = R.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void *args[] = {&R.RA};
+  CK(cudaLaunchKernelExC(&cfg, R.res_kernel, args));
+  CK(cudaEventRecord(R.ev_done, R.stream));
+  return OPM_OK;
+}
 
 opm_status runner_create(const std::vector<opm_solver *> &mem, cudaStream_t stream, const opm_options &o,
                          Runner **out) {
@@ -651,6 +792,9 @@ opm_status runner_create(const std::vector<opm_solver *> &mem, cudaStream_t stre
   R->cp_sweeps = o.cp_sweeps;
   R->tri_sweeps = o.tri_sweeps;
   R->reuse = product_reuse_applies(o, R->fp32);
+  int ntree = 0;
+  for (auto *h : mem) ntree += tree_order(*R, h);
+  R->tree = ntree == 0 ? kTreeNone : ntree == R->nsys ? kTreeAll : kTreeMixed;
   // second buffers of the iterative sweeps, kept by the members
   for (auto *h : mem) {
     opm_status sa = OPM_OK;
@@ -789,7 +933,8 @@ opm_status runner_create(const std::vector<opm_solver *> &mem, cudaStream_t stre
         return fail(OPM_ERR_CUDA);
       }
   }
-  if ((s = build_graphs(*R)) != OPM_OK) return fail(s);
+  if (sweep_launch == OPM_SWEEP_AUTO && !profile && (s = resident_create(*R, max_entries)) != OPM_OK) return fail(s);
+  if (!R->resident && (s = build_graphs(*R)) != OPM_OK) return fail(s);
   if (cudaStreamSynchronize(stream) != cudaSuccess) {
     cudaGetLastError();
     return fail(OPM_ERR_CUDA);
@@ -805,6 +950,10 @@ opm_status runner_sync_wells(Runner &R) {
   bool any = false;
   for (auto *h : R.mem) any = any || h->sys.nwells > 0;
   if (any == R.has_wells) return OPM_OK;
+  if (R.resident) {  // no graphs: the kernel looks at the wells itself
+    R.has_wells = any;
+    return OPM_OK;
+  }
   CK(cudaStreamSynchronize(R.stream));
   if (R.solve_exec) cudaGraphExecDestroy(R.solve_exec);
   if (R.iter_exec) cudaGraphExecDestroy(R.iter_exec);
@@ -820,6 +969,7 @@ opm_status runner_push(Runner &R) {
   if (ws != OPM_OK) return ws;
   for (int s = 0; s < R.nsys; ++s) {
     R.h_sys[s] = R.mem[s]->sys;
+    R.h_sys[s].tree = tree_order(R, R.mem[s]);
     if (!R.reuse) R.h_sys[s].uz = nullptr;
   }
   CK(cudaMemcpyAsync((void *)R.B.sys, R.h_sys, sizeof(Sys) * R.nsys, cudaMemcpyHostToDevice, R.stream));
@@ -833,6 +983,7 @@ opm_status runner_pull_results(Runner &R) {
 
 // Enqueue (no host wait): optional factorisation, then an optional solve.
 opm_status runner_enqueue(Runner &R, bool factor, bool solve) {
+  if (R.resident) return resident_enqueue(R, factor, solve);
   opm_status s = runner_push(R);
   if (s != OPM_OK) return s;
   if (factor && solve && R.fs_exec) {
@@ -853,6 +1004,7 @@ opm_status runner_wait(Runner &R) {
 
 // Kernel launches of one solve-graph execution, for the launch counter.
 int64_t solve_graph_launches(const Runner &R) {
+  if (R.resident) return 1;
   int maxit = 1;
   for (int s = 0; s < R.nsys; ++s) maxit = std::max(maxit, R.h_res[s].iters);
   const int64_t bodies = (maxit + R.chunk - 1) / R.chunk;

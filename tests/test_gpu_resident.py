@@ -1,0 +1,97 @@
+"""The resident kernel (one cooperative launch per refactorisation and solve:
+sweep_launch "auto" on a single system) against the launches per phase: the
+same arithmetic in the same order, so factors, solutions, iteration counts
+and residuals are compared bitwise, at the edges of its units (32-row slices,
+256- and 1024-row tiles, 8,192-row groups) and of its two forms."""
+import numpy as np
+import pytest
+
+from paper_2309_11488_gb300 import opm, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def grid(nx, ny, nz, seed=3):
+    logk = np.random.default_rng(seed).normal(size=(nz, ny, nx))
+    return synth.grid_system(nx, ny, nz, logk, seed=synth.SEED_BASE + seed)
+
+
+def both_forms(s, precision, rtol, schedule="auto", part=None, wells=None, reuse=0, refactor=True):
+    """(factors, x, status, iters, relres) with launches per phase and resident."""
+    b = dev(s.x_true)  # any right-hand side does
+    vals2 = dev(s.vals * (1.0 + 0.01 * np.cos(np.arange(s.nnzb)))[:, None])
+    out = []
+    for sweep in ("per_phase", "auto"):
+        with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), dev(s.vals), schedule=schedule, precision=precision,
+                        sweep_launch=sweep, part=part, product_reuse=reuse) as sv:
+            if wells is not None:
+                assert sv.set_wells(wells) == opm.OPM_OK
+            x = torch.full_like(b, 7.0)
+            if refactor:
+                sv.launch(vals2, b, x, rtol=rtol)
+                st, it, rr = sv.wait()
+            else:
+                _, st, it, rr = sv.solve(b, x, rtol=rtol)
+            x2, st2, it2, rr2 = sv.solve(b, rtol=1e-2, maxit=3)  # again, on the kept factors
+            out.append((*sv.factors(), x.cpu().numpy(), x2.cpu().numpy(), np.array([st, it, rr, st2, it2, rr2])))
+    for a, c in zip(*out):
+        np.testing.assert_array_equal(a, c)
+    assert out[0][-1][0] == 0
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 257, 1023, 1025, 8191, 8193])
+def test_edges_of_units(n, precision):
+    both_forms(synth.chain_system(n), precision, 1e-8, schedule="colour")
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("dims", [(39, 39, 40), (41, 39, 40), (68, 67, 68), (69, 67, 68)])
+def test_edges_of_forms(dims, precision):
+    # 60,800 rows: the last size of the three-warp form on 152 SMs; 311,296: the last of the resident kernel
+    both_forms(grid(*dims), precision, 1e-3)
+
+
+@pytest.mark.parametrize("schedule", ["natural", "level", "colour", "colour_kempe"])
+def test_schedules_and_long_rows(schedule):
+    # rows past the blocks loaded ahead, non-symmetric pattern; long dependency chains in natural order
+    s = synth.one_way_system(synth.random_pattern_system(700, 9, 11), 0.3, 12)
+    both_forms(s, "fp64", 1e-10, schedule=schedule)
+
+
+@pytest.mark.parametrize("n", [14, 42])  # three-warp and one-warp form
+@pytest.mark.parametrize("case", ["jacobi_wells", "wells", "plain_product", "solve_only"])
+def test_options(n, case):
+    s = synth.config3(n)
+    part = synth.partition_grid(s, 5) if case == "jacobi_wells" else None
+    wells = synth.wells(s, 9, 4) if "wells" in case else None
+    both_forms(s, "fp64", 1e-6, part=part, wells=wells, reuse=-1 if case == "plain_product" else 0,
+               refactor=case != "solve_only")
+
+
+def test_bounded_wait_expires_and_singular_pivot():
+    s = synth.config2()
+    st, h = opm.opm_bsr_create(s.nb, s.rowptr, s.colidx, s.vals,
+                               opm.opm_options_default(spin_limit_us=20000, debug_skip_item=3), check=False)
+    assert st == opm.OPM_ERR_TIMEOUT
+    opm.opm_destroy(h)
+    rows = np.repeat(np.arange(s.nb), np.diff(s.rowptr))
+    bad = s.vals.copy()
+    bad[np.flatnonzero(rows == s.colidx)[5]] = 0.0
+    b = dev(s.x_true)
+    with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), dev(s.vals)) as sv:
+        x0, st0, it0, rr0 = sv.solve(b)
+        x = torch.empty_like(b)
+        sv.launch(dev(bad), b, x)
+        st, it, rr = sv.wait()
+        assert st == opm.OPM_ERR_ZERO_PIVOT and (x == 0).all() and np.isnan(rr)
+        assert sv.factor(dev(bad)) == opm.OPM_ERR_ZERO_PIVOT and opm.opm_last_error_row(sv.h) == 5
+        assert sv.factor(dev(s.vals)) == opm.OPM_OK  # recovers
+        x1, st1, it1, rr1 = sv.solve(b)
+        assert (st1, it1, rr1) == (st0, it0, rr0) and torch.equal(x1, x0)
