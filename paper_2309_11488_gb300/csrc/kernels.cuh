@@ -501,6 +501,35 @@ __device__ __forceinline__ void row_operator(const Sys &S, const double *__restr
   row_spmv(S.a_rp, S.a_col, S.a_val, x, i, S.n, y0, y1, y2);
 }
 
+// row_operator without wells on x = b_in in the caller's order: block j's
+// vector is x[perm[j]].
+__device__ __forceinline__ void row_operator_gather(const Sys &S, int i, double &y0, double &y1, double &y2) {
+  const int lane = threadIdx.x & 31, n = S.n, s0 = i - lane;
+  const int len = (i < n) ? __ldg(S.a_rp + i + 1) - __ldg(S.a_rp + i) : 0;
+  int base = (s0 < n) ? __ldg(S.a_rp + s0) : 0;
+  const int maxlen = __reduce_max_sync(0xffffffffu, len);
+  const unsigned lt = lanemask_lt();
+  const double *__restrict__ x = S.b_in;
+  const double *__restrict__ val = S.a_val;
+  for (int k = 0; k < maxlen; ++k) {
+    const unsigned m = __ballot_sync(0xffffffffu, len > k);
+    if (len > k) {
+      const int cnt = __popc(m);
+      const int q = __popc(m & lt);
+      const int j = __ldg(S.perm + __ldcs(S.a_col + base + q));
+      const double *a = val + 9ll * base + q;
+      const double x0 = __ldg(x + 3ll * j), x1 = __ldg(x + 3ll * j + 1), x2 = __ldg(x + 3ll * j + 2);
+      const double a0 = __ldcs(a), a1 = __ldcs(a + cnt), a2 = __ldcs(a + 2 * cnt);
+      const double a3 = __ldcs(a + 3 * cnt), a4 = __ldcs(a + 4 * cnt), a5 = __ldcs(a + 5 * cnt);
+      const double a6 = __ldcs(a + 6 * cnt), a7 = __ldcs(a + 7 * cnt), a8 = __ldcs(a + 8 * cnt);
+      y0 = fma(a0, x0, fma(a1, x1, fma(a2, x2, y0)));
+      y1 = fma(a3, x0, fma(a4, x1, fma(a5, x2, y1)));
+      y2 = fma(a6, x0, fma(a7, x1, fma(a8, x2, y2)));
+    }
+    base += __popc(m);
+  }
+}
+
 // y += the first lead blocks of lane's row i of A's warp-sliced layout
 // (FP64).  The slab layout is walked with every row's full length; lanes
 // issue loads only for their first lead blocks, and the walk stops after
@@ -873,17 +902,34 @@ __global__ void __launch_bounds__(256, 8) k_finish(Batch B) {
   }
 }
 
-// y = A x in the caller's order (x already permuted into w).
-__global__ void __launch_bounds__(256, 8) k_spmv_plain(Batch B) {
-  OPM_TILE_S(B, S, lt);
-  const int i = lt * kSpmvRows + threadIdx.x;
+// y = A x for one system, whose descriptor is the kernel's parameter (a copy
+// to the device ahead of the launch would cost more than a small product).
+// GATHER: x is read in the caller's order through perm; otherwise w holds it.
+template <bool GATHER>
+__global__ void __launch_bounds__(256, 8) k_spmv_plain(const __grid_constant__ Sys S) {
+  pdl_enter();
+  const int i = blockIdx.x * kSpmvRows + threadIdx.x;
   double y0 = 0.0, y1 = 0.0, y2 = 0.0;
-  row_operator(S, S.w, i, y0, y1, y2);
+  if (GATHER) row_operator_gather(S, i, y0, y1, y2);
+  else row_operator(S, S.w, i, y0, y1, y2);
   if (i < S.n) {
     const int o = S.perm[i];
     S.x_out[3ll * o] = y0;
     S.x_out[3ll * o + 1] = y1;
     S.x_out[3ll * o + 2] = y2;
+  }
+}
+
+// w[i] = b_in[perm[i]] for one system (its descriptor the parameter).
+__global__ void __launch_bounds__(256, 6) k_gather_one(const __grid_constant__ Sys S) {
+  pdl_trigger();
+  const int lt = blockIdx.x;
+  OPM_TILE_ROWS(i, lt) {
+    if (i < S.n) {
+      const int o = S.perm[i];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) S.w[3ll * i + c] = S.b_in[3ll * o + c];
+    }
   }
 }
 

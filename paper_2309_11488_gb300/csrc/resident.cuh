@@ -32,7 +32,7 @@
 
 namespace opm {
 
-enum ResidentWork { kResFactor = 1, kResSolve = 2 };
+enum ResidentWork { kResFactor = 1, kResSolve = 2, kResApply = 4 };
 
 // Device words of one runner, zero between launches: the CTA that leaves
 // last clears them.
@@ -313,14 +313,16 @@ __device__ __forceinline__ Vec3<TF> sweep_gather(const void *y, const double *z,
 }
 
 // One slice of a sweep over the phase's rows [E.z, E.w): fwd_rows (fwd; the
-// right-hand side p in the first half of an iteration, s in the second) or
-// bwd_rows.
-template <typename TF>
+// right-hand side p in the first half of an iteration, s in the second, the
+// caller's vector in a standalone application) or bwd_rows.  A standalone
+// application reads and writes the caller's order in place.
+template <typename TF, int MODE>
 __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool second) {
   const Sys &S = c.sm.sys[E.x];
   const int lane = c.lane, sl = E.y, s0 = sl * 32, i = s0 + lane;
+  constexpr bool kPlain = MODE == kModePlain;
   TF *y = static_cast<TF *>(S.y);
-  double *z = second ? S.sh : S.ph;
+  double *z = kPlain ? S.t : second ? S.sh : S.ph;
   const uint2 M = __ldg(S.sl_mask + sl);
   const bool eager = (M.x >> lane) & 1u;
   const bool act = i >= E.z && i < E.w && (fwd || !eager);
@@ -331,7 +333,11 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
   int base = __ldg(rp + s0);
   const int maxlen = __reduce_max_sync(0xffffffffu, len);
   Vec3<TF> a{TF(0), TF(0), TF(0)};
-  if (act && fwd) {
+  const int64_t o = kPlain && act ? 3ll * __ldg(S.perm + i) : 0;
+  if (act && fwd && kPlain) {
+    const Vec3<double> h = load3cg(S.b_in + o);
+    a = {(TF)h.c0, (TF)h.c1, (TF)h.c2};
+  } else if (act && fwd) {
     Vec3<double> h = load3cg(S.r + 3ll * i);
     const Vec3<double> vo = load3cg(S.v + 3ll * i);
     const Scal &sc = c.sm.sc[E.x];
@@ -373,7 +379,7 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
     }
   }
   if (!act) return;
-  if (!fwd && sizeof(TF) == sizeof(double) && S.uz && ((__ldg(S.sp_mask + sl).y >> lane) & 1u)) {
+  if (!kPlain && !fwd && sizeof(TF) == sizeof(double) && S.uz && ((__ldg(S.sp_mask + sl).y >> lane) & 1u)) {
     const Vec3<TF> yr = load3cg(static_cast<const TF *>(y) + 3ll * i);
     double *w = S.uz + 3ll * i;
     w[0] = (double)(yr.c0 - a.c0);
@@ -384,6 +390,7 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
     TF d[9];
     load_dinv<TF>(lu + S.d_off + (int64_t)kSliceVals * sl + lane, d);
     store_dinv_product<TF>(z + 3ll * i, d, a.c0, a.c1, a.c2);
+    if (kPlain) store_dinv_product<TF>(S.x_out + o, d, a.c0, a.c1, a.c2);
   }
   if (fwd && ((M.y >> lane) & 1u)) {
     TF *yi = y + 3ll * i;
@@ -602,12 +609,13 @@ __device__ __forceinline__ int preload_row(const int32_t *col, const T *vals, in
 }
 
 // sweep_unit by a trio; FIRST: wait() is called here.
-template <typename TF, bool FIRST>
+template <typename TF, int MODE, bool FIRST>
 __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool second) {
   const Sys &S = c.sm.sys[E.x];
   const int lane = c.lane, r = c.r, sl = E.y, s0 = sl * 32, i = s0 + lane;
+  constexpr bool kPlain = MODE == kModePlain;
   TF *y = static_cast<TF *>(S.y);
-  double *z = second ? S.sh : S.ph;
+  double *z = kPlain ? S.t : second ? S.sh : S.ph;
   const uint2 M = __ldg(S.sl_mask + sl);
   const bool eager = (M.x >> lane) & 1u;
   const bool act = i >= E.z && i < E.w && (fwd || !eager);
@@ -631,9 +639,11 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   if (FIRST) c.wait();
   double h = 0.0, vo = 0.0, po = 0.0;
   TF a = TF(0);
-  const int64_t e = 3ll * i + r;
+  const int64_t e = 3ll * i + r, o = kPlain && act ? 3ll * __ldg(S.perm + i) + r : 0;
   if (act) {
-    if (fwd) {
+    if (fwd && kPlain) {
+      h = __ldcg(S.b_in + o);
+    } else if (fwd) {
       h = __ldcg(S.r + e);
       vo = __ldcg(S.v + e);
       if (!second) po = __ldcg(S.p + e);
@@ -648,7 +658,9 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
     if (lead > k) vv[k] = sweep_gather<TF>(S.y, z, fwd, jp[k]);
   }
   const TF y0 = a;  // the backward sweep's y_i
-  if (act && fwd) {
+  if (act && fwd && kPlain) {
+    a = (TF)h;
+  } else if (act && fwd) {
     const Scal &sc = c.sm.sc[E.x];
     h = second ? fma(-sc.alpha, vo, h) : fma(sc.beta, fma(-sc.omega, vo, po), h);
     (second ? S.s : S.p)[e] = h;
@@ -676,9 +688,13 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   c.trio_sync();
   const TF a0 = (TF)ex[0][lane], a1 = (TF)ex[1][lane], a2 = (TF)ex[2][lane];
   if (!act) return;
-  if (!fwd && sizeof(TF) == sizeof(double) && S.uz && ((__ldg(S.sp_mask + sl).y >> lane) & 1u))
+  if (!kPlain && !fwd && sizeof(TF) == sizeof(double) && S.uz && ((__ldg(S.sp_mask + sl).y >> lane) & 1u))
     S.uz[e] = (double)(y0 - a);
-  if (use_d) z[e] = (double)fma(d[0], a0, fma(d[1], a1, d[2] * a2));
+  if (use_d) {
+    const double v = (double)fma(d[0], a0, fma(d[1], a1, d[2] * a2));
+    z[e] = v;
+    if (kPlain) S.x_out[o] = v;
+  }
   if (fwd && ((M.y >> lane) & 1u)) y[e] = a;
 }
 
@@ -733,14 +749,13 @@ __device__ __forceinline__ void product_trio(ResCtx &c, int4 E, int step, bool r
     }
     base += __popc(m);
   }
-  if (in) {
-    if (fin) S.x_out[3ll * o + r] = ok ? __ldcg(S.x + e) : 0.0;
-    else io.out[e] = y;
-  }
+  if (in && !fin) io.out[e] = y;
   double(*ex)[32] = c.sm.ex[c.trio][c.flip][0];
   c.flip ^= 1;
   ex[r][lane] = y;
   c.trio_sync();
+  // past the trio's reads of b: x may be written in its place
+  if (in && fin) S.x_out[3ll * o + r] = ok ? __ldcg(S.x + e) : 0.0;
   // the dot products, one per warp: (q, y), (y, y), (q, q)
   if (r > 0 && step != kStepS) return;
   double v[1] = {0.0};
@@ -978,31 +993,48 @@ __device__ __forceinline__ void resident_factor(ResCtx &c) {
   __syncthreads();
 }
 
-// The sweep of a phase's entries.
-template <typename TF, bool TRIO>
-__device__ __forceinline__ void sweep_stage(ResCtx &c, int e0, int e1, bool fwd, bool second) {
-  stage(c, e0, e1, [&](int e, auto first) {
-    constexpr bool F = decltype(first)::value;
-    const int4 E = __ldg(c.R.B.ent + e);
-    const bool run = c.runs(E.x);
-    if (F && (!TRIO || !run)) c.wait();
-    if (!run) return;
-    if constexpr (TRIO) sweep_trio<TF, F>(c, E, fwd, second);
-    else sweep_unit<TF>(c, E, fwd, second);
-  });
+// One preconditioner application.  The first forward phase follows the
+// caller's wait; the last phase ends with an arrival.
+template <typename TF, int MODE, bool TRIO>
+__device__ __forceinline__ void resident_apply(ResCtx &c, bool second) {
+  const Batch &B = c.R.B;
+  // the first phase's rows have no L blocks: nothing to load ahead
+#pragma unroll 1
+  for (int e = __ldg(B.fwd_ptr) + c.g, e1 = __ldg(B.fwd_ptr + 1); e < e1; e += c.W) {
+    const int4 E = __ldg(B.ent + e);
+    if (!c.runs(E.x)) continue;
+    if constexpr (TRIO) sweep_trio<TF, MODE, false>(c, E, true, second);
+    else sweep_unit<TF, MODE>(c, E, true, second);
+  }
+  c.arrive();
+  // forward phases 1 .. np - 1, then backward phases np - 1 .. 0
+  const int np = B.nphases;
+#pragma unroll 1
+  for (int q = 1; q < 2 * np && !c.dead; ++q) {
+    const bool fwd = q < np;
+    const int32_t *ptr = fwd ? B.fwd_ptr + q : B.bwd_ptr + (2 * np - 1 - q);
+    const int e0 = __ldg(ptr), e1 = __ldg(ptr + 1);
+    if (!fwd && e0 == e1) continue;
+    stage(c, e0, e1, [&](int e, auto first) {
+      constexpr bool F = decltype(first)::value;
+      const int4 E = __ldg(B.ent + e);
+      const bool run = c.runs(E.x);
+      if (F && (!TRIO || !run)) c.wait();
+      if (!run) return;
+      if constexpr (TRIO) sweep_trio<TF, MODE, F>(c, E, fwd, second);
+      else sweep_unit<TF, MODE>(c, E, fwd, second);
+    });
+  }
 }
 
-// TF: factor precision; TRIO: three warps per slice (with one warp more for
-// the barrier) or one; NT: threads per CTA, one CTA per SM.
-template <typename TF, bool TRIO, int NT>
-__global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resident R) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  ResShared &sm = *reinterpret_cast<ResShared *>(smem_raw);
+// The start of a launch: descriptors and scalars into shared memory, and the
+// warp's place among the units.
+template <bool TRIO>
+__device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &sm) {
   const Batch &B = R.B;
-  const int wp = threadIdx.x >> 5;
-  ResCtx c{R, sm, (int)(threadIdx.x & 31), wp, NT / 32, 0, 0, 0, 0, 0, 0u, false, threadIdx.x == NT - 32};
+  const int wp = threadIdx.x >> 5, nt = blockDim.x;
+  ResCtx c{R, sm, (int)(threadIdx.x & 31), wp, nt / 32, 0, 0, 0, 0, 0, 0u, false, (int)threadIdx.x == nt - 32};
   if (TRIO) {
-    static_assert(!TRIO || NT == kTrioThreads, "the trios and one warp more");
     c.r = wp % 3;
     c.trio = wp / 3;
     c.g = c.trio < kTrios ? c.trio * gridDim.x + blockIdx.x : 0x40000000;  // the last warp takes no units
@@ -1011,26 +1043,90 @@ __global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resi
     c.g = c.warp_id();  // consecutive units go to different SMs
     c.W = c.warps();
   }
-  // ---- descriptors and scalars of this CTA
-  {
-    const int4 *src = reinterpret_cast<const int4 *>(B.nsys == 1 ? &R.one : B.sys);
-    int4 *dst = reinterpret_cast<int4 *>(sm.sys);
-    static_assert(sizeof(Sys) % sizeof(int4) == 0, "descriptors are copied in 16-byte pieces");
-    for (int q = threadIdx.x; q < B.nsys * (int)(sizeof(Sys) / sizeof(int4)); q += NT) dst[q] = src[q];
-  }
+  const int4 *src = reinterpret_cast<const int4 *>(B.nsys == 1 ? &R.one : B.sys);
+  int4 *dst = reinterpret_cast<int4 *>(sm.sys);
+  static_assert(sizeof(Sys) % sizeof(int4) == 0, "descriptors are copied in 16-byte pieces");
+  for (int q = threadIdx.x; q < B.nsys * (int)(sizeof(Sys) / sizeof(int4)); q += nt) dst[q] = src[q];
   __syncthreads();
-  const bool factor = R.work & kResFactor, solve = R.work & kResSolve;
   if (threadIdx.x < B.nsys) {
     Scal z{};
     const Sys &S = sm.sys[threadIdx.x];
     z.tol = S.rtol;
     z.maxit = S.maxit;
     // an earlier factorisation's failure makes the solve fail
-    const int32_t ferr = (solve && !factor && !S.skip) ? S.st->ferror : 0;
+    const int32_t ferr = (R.work == kResSolve && !S.skip) ? S.st->ferror : 0;
     z.status = ferr != 0 ? ferr : S.skip ? OPM_OK : kRunning;
     sm.sc[threadIdx.x] = z;
   }
   __syncthreads();
+  return c;
+}
+
+// The end: the last CTA to leave writes the outcome and clears the device words.
+__device__ __forceinline__ void resident_leave(ResCtx &c) {
+  const Resident &R = c.R;
+  ResShared &sm = c.sm;
+  const bool factor = R.work & kResFactor, solve = R.work & kResSolve;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    sm.last = atomicAdd(&R.ctl->exits, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!sm.last) return;
+  const bool aborted = ld_acquire(&R.ctl->abort) != 0u;
+  for (int s = threadIdx.x; s < R.B.nsys; s += blockDim.x) {
+    const Sys &S = sm.sys[s];
+    const Scal &sc = sm.sc[s];
+    if (!S.skip) {
+      const int32_t ferr = __ldcg(R.err + 2 * s);
+      DevState *st = S.st;
+      Result r{};
+      r.status = aborted ? (int32_t)OPM_ERR_TIMEOUT : solve ? sc.status : ferr;  // 0 after an application
+      r.iters = sc.iters;
+      r.relres = aborted ? nan("") : sc.relres;
+      r.err_row = ferr != 0 ? 0x7fffffff - __ldcg(R.err + 2 * s + 1) : 0x7fffffff;
+      if (factor) {
+        st->ferror = aborted ? (int32_t)OPM_ERR_TIMEOUT : ferr;
+        st->err_row = r.err_row;
+      }
+      if (factor || solve) {
+        st->error = aborted ? (int32_t)OPM_ERR_TIMEOUT : 0;
+        st->status = r.status;
+      }
+      R.res[s] = r;
+    }
+    R.err[2 * s] = 0;
+    R.err[2 * s + 1] = 0;
+  }
+  if (threadIdx.x == 0) {
+    R.ctl->arrive = 0;
+    R.ctl->exits = 0;
+    R.ctl->abort = 0;
+  }
+}
+
+// A standalone application z = inv(LU) r (opm_ilu_apply).
+template <typename TF, bool TRIO, int NT>
+__global__ void __launch_bounds__(NT, 1) k_resident_apply(const __grid_constant__ Resident R) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  ResCtx c = resident_enter<TRIO>(R, *reinterpret_cast<ResShared *>(smem_raw));
+  resident_apply<TF, kModePlain, TRIO>(c, false);
+  resident_leave(c);
+}
+
+// Factorisation and solve.  TF: factor precision; TRIO: three warps per slice
+// (with one warp more for the barrier) or one; NT: threads per CTA, one CTA
+// per SM.
+template <typename TF, bool TRIO, int NT>
+__global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resident R) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  ResShared &sm = *reinterpret_cast<ResShared *>(smem_raw);
+  const Batch &B = R.B;
+  static_assert(!TRIO || NT == kTrioThreads, "the trios and one warp more");
+  ResCtx c = resident_enter<TRIO>(R, sm);
+  const bool factor = R.work & kResFactor, solve = R.work & kResSolve;
   bool wells = false, reuse = false;
   for (int s = 0; s < B.nsys; ++s) {
     wells = wells || (sm.sys[s].nwells > 0 && !sm.sys[s].skip);
@@ -1063,24 +1159,7 @@ __global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resi
     } else if (step != kStepSetup) {
       const bool second = step == kStepS;
       if (step != kStepFinish) {
-        // the first phase's rows have no L blocks: nothing to load ahead
-#pragma unroll 1
-        for (int e = __ldg(B.fwd_ptr) + c.g, e1 = __ldg(B.fwd_ptr + 1); e < e1; e += c.W) {
-          const int4 E = __ldg(B.ent + e);
-          if (!c.runs(E.x)) continue;
-          if constexpr (TRIO) sweep_trio<TF, false>(c, E, true, second);
-          else sweep_unit<TF>(c, E, true, second);
-        }
-        c.arrive();
-        // forward phases 1 .. np - 1, then backward phases np - 1 .. 0
-        const int np = B.nphases;
-#pragma unroll 1
-        for (int q = 1; q < 2 * np && !c.dead; ++q) {
-          const bool fwd = q < np;
-          const int32_t *ptr = fwd ? B.fwd_ptr + q : B.bwd_ptr + (2 * np - 1 - q);
-          const int e0 = __ldg(ptr), e1 = __ldg(ptr + 1);
-          if (fwd || e0 != e1) sweep_stage<TF, TRIO>(c, e0, e1, fwd, second);
-        }
+        resident_apply<TF, kModeP, TRIO>(c, second);
       } else {
         c.arrive();
       }
@@ -1104,43 +1183,7 @@ __global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resi
     step = !any ? kStepFinish : step == kStepP ? kStepS : step == kStepS ? kStepUpdate : kStepP;
   }
 
-  // ---- leave: the last CTA writes the outcome and clears the device words
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    sm.last = atomicAdd(&R.ctl->exits, 1u) == gridDim.x - 1;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!sm.last) return;
-  const bool aborted = ld_acquire(&R.ctl->abort) != 0u;
-  for (int s = threadIdx.x; s < B.nsys; s += NT) {
-    const Sys &S = sm.sys[s];
-    const Scal &sc = sm.sc[s];
-    if (!S.skip) {
-      const int32_t ferr = __ldcg(R.err + 2 * s);
-      DevState *st = S.st;
-      Result r{};
-      r.status = aborted ? (int32_t)OPM_ERR_TIMEOUT : solve ? sc.status : ferr;
-      r.iters = sc.iters;
-      r.relres = aborted ? nan("") : sc.relres;
-      r.err_row = ferr != 0 ? 0x7fffffff - __ldcg(R.err + 2 * s + 1) : 0x7fffffff;
-      if (factor) {
-        st->ferror = aborted ? (int32_t)OPM_ERR_TIMEOUT : ferr;
-        st->err_row = r.err_row;
-      }
-      st->error = aborted ? (int32_t)OPM_ERR_TIMEOUT : 0;
-      st->status = r.status;
-      R.res[s] = r;
-    }
-    R.err[2 * s] = 0;
-    R.err[2 * s + 1] = 0;
-  }
-  if (threadIdx.x == 0) {
-    R.ctl->arrive = 0;
-    R.ctl->exits = 0;
-    R.ctl->abort = 0;
-  }
+  resident_leave(c);
 }
 
 }  // namespace opm

@@ -95,3 +95,29 @@ def test_bounded_wait_expires_and_singular_pivot():
         assert sv.factor(dev(s.vals)) == opm.OPM_OK  # recovers
         x1, st1, it1, rr1 = sv.solve(b)
         assert (st1, it1, rr1) == (st0, it0, rr0) and torch.equal(x1, x0)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("n", [8, 14, 42, 70])  # three-warp, one-warp form, launches per phase
+def test_operators_alone_and_in_place(n, precision):
+    """Product and application against the launches per phase, also with the output over the input (at an offset
+    too), and a solve whose x takes b's place."""
+    s = synth.config3(n)
+    x = dev(s.x_true)
+    n3 = x.numel()
+    out = []
+    for sweep in ("per_phase", "auto"):
+        with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), dev(s.vals), precision=precision, sweep_launch=sweep) as sv:
+            y, z = sv.spmv(x), sv.ilu_apply(x)
+            for op, ref in ((sv.spmv, y), (sv.ilu_apply, z)):
+                for shift in (0, 3):
+                    buf = torch.zeros(n3 + 3, dtype=torch.float64, device="cuda")
+                    buf[:n3] = x
+                    assert torch.equal(op(buf[:n3], buf[shift:shift + n3]), ref)
+            a, st, it, rr = sv.solve(y, rtol=1e-4)
+            b = y.clone()
+            a2, st2, it2, rr2 = sv.solve(b, b, rtol=1e-4)
+            assert (st, it, rr) == (st2, it2, rr2) and torch.equal(a, a2)
+            out.append((y, z, a))
+    for u, v in zip(*out):
+        assert torch.equal(u, v)
