@@ -101,9 +101,12 @@ enum {
   OPM_SWEEP_AUTO = 0,        /* a single system of up to about 300,000 rows:
                                 one cooperative launch that refactors and
                                 solves it, with bounded grid barriers between
-                                its stages; otherwise per-phase launches up
-                                to 1024 phases, cooperative sweeps past that.
-                                Every form gives the same bits              */
+                                its stages (on a stream other than the default
+                                one, up to about 18,000 rows and on a quarter
+                                of the SMs, so that streams overlap);
+                                otherwise per-phase launches up to 1024
+                                phases, cooperative sweeps past that.  Every
+                                form gives the same bits                    */
   OPM_SWEEP_PER_PHASE = 1,   /* one kernel launch per phase                 */
   OPM_SWEEP_COOPERATIVE = 2  /* one cooperative launch walking all phases,
                                 with a bounded grid barrier between them    */

@@ -630,6 +630,20 @@ void runner_destroy(Runner *R) {
 bool resident_trios(int nslices, int sms) { return 2 * (int64_t)nslices <= 5 * (int64_t)kTrios * sms; }
 bool resident_size(int nslices, int sms) { return nslices <= 2 * (kResidentThreads / 32) * (int64_t)sms; }
 
+// A handle or batch on a stream of its own (not the default stream) is taken
+// to share the device with others.  A resident launch over all SMs would make
+// theirs wait for its whole solve, so it takes a quarter of the SMs, up to
+// three slices per trio (18,240 rows on 152 SMs); larger systems keep the
+// launches per phase, which overlap.  us per solve (FP64, rtol 1e-2) with 1, 2,
+// 4 and 8 handles on as many streams, launches per phase / all SMs / a quarter:
+//    3,868 rows  627 334 202 180 / 390 382 380 379 /  401 207 108 103
+//    7,574 rows  872 485 279 258 / 457 453 450 449 /  582 297 152 150
+//   18,671 rows  961 600 370 322 / 531 520 522 534 /  947 487 258 257
+//   44,431 rows  898 689 439 379 / 605 615 615 612 / 1604 844 438 435
+//  249,053 rows 2208 1522 1121 1121 / 1698 1691 1683 1684 / 4542 2321 1203 1200
+int quarter(int sms) { return (sms + 3) / 4; }
+bool shares_device(int nslices, int sms) { return nslices <= 3 * kTrios * quarter(sms); }
+
 // A system's order of summation follows from its size and the sweeps alone,
 // so it is the same in every launch form, alone and in a batch.
 int32_t tree_order(const Runner &R, const opm_solver *h) {
@@ -662,6 +676,7 @@ const void *resident_kernel(bool trio, bool apply) {
 // Whether the runner's system goes to the resident kernel, and its work lists.
 opm_status resident_create(Runner &R, int max_entries) {
   if (R.nsys > 1 || R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(R.nall, R.sms)) return OPM_OK;
+  if (R.stream && !shares_device(R.nall, R.sms)) return OPM_OK;
   const bool trio = resident_trios(R.nall, R.sms);
   R.res_kernel = R.fp32 ? resident_kernel<float>(trio, false) : resident_kernel<double>(trio, false);
   R.res_apply = R.fp32 ? resident_kernel<float>(trio, true) : resident_kernel<double>(trio, true);
@@ -675,7 +690,8 @@ opm_status resident_create(Runner &R, int max_entries) {
       return OPM_OK;
     }
   }
-  R.res_grid = std::max(1, std::min(R.sms, std::max(max_entries, R.nall)));  // one CTA per SM
+  const int sms = R.stream ? quarter(R.sms) : R.sms;  // one CTA per SM
+  R.res_grid = std::max(1, std::min(sms, std::max(max_entries, R.nall)));
   std::vector<int32_t> off_s(1, 0), off_u(1, 0), goff_s(1, 0), goff_u(1, 0);
   std::vector<int2> grp_s, grp_u;
   for (int s = 0; s < R.nsys; ++s) {

@@ -121,3 +121,32 @@ def test_operators_alone_and_in_place(n, precision):
             out.append((y, z, a))
     for u, v in zip(*out):
         assert torch.equal(u, v)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("dims", [(33, 1, 1), (20, 20, 20), (32, 30, 19), (32, 571, 1)])
+def test_handles_on_streams_of_their_own(dims, precision):
+    """Three handles refactor and solve at once, each on a stream of its own, which bounds the resident kernel's grid
+    and sizes (18,240 rows: the last on 152 SMs): the bits of the launches per phase on the default stream."""
+    s = grid(*dims)
+    vals = [dev(s.vals * (1.0 + 0.01 * k * np.cos(np.arange(s.nnzb)))[:, None]) for k in range(3)]
+    b = dev(s.x_true)
+    an = opm.Analysis(s.nb, s.rowptr, s.colidx)
+    want = []
+    for v in vals:
+        with opm.Solver.from_analysis(an, v, precision=precision, sweep_launch="per_phase") as sv:
+            want.append((*sv.solve(b, rtol=1e-3), sv.ilu_apply(b)))
+    streams = [torch.cuda.Stream() for _ in vals]
+    torch.cuda.synchronize()
+    sv = [opm.Solver.from_analysis(an, vals[0], precision=precision, stream=q) for q in streams]
+    xs = [torch.empty_like(b) for _ in vals]
+    torch.cuda.synchronize()
+    for h, v, x in zip(sv, vals, xs):
+        h.launch(v, b, x, rtol=1e-3)
+    for h, x, (xw, st, it, rr, z) in zip(sv, xs, want):
+        assert h.wait() == (st, it, rr) and torch.equal(x, xw)
+        out = torch.empty_like(b)
+        torch.cuda.synchronize()
+        h.ilu_apply(b, out)
+        assert torch.equal(out, z)
+        h.close()
