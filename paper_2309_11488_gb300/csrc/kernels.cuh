@@ -77,6 +77,7 @@ struct alignas(16) Sys {
   int64_t u_off, d_off;
   double *x, *r, *rh, *p, *v, *ph, *s, *sh, *t, *w;
   void *y;   // forward intermediate (factor precision)
+  float *zf; // FP32 factors: z as floats, for the resident kernel's backward gathers
   void *y2;  // Jacobi triangular sweeps (tri_sweeps > 0): second forward iterate, else NULL
   double *z2;  // Jacobi triangular sweeps: second backward iterate, else NULL
   double *partials;      // per tile: up to 4 partial sums

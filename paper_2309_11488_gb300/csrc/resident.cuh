@@ -304,12 +304,20 @@ __device__ __forceinline__ void finish_dot(ResCtx &c, int step) {
 // The wide form: a lane per row, as in the launch-per-phase kernels.  The
 // caller has waited.
 
-// The earlier phases' results for a sweep: y (forward) or z (backward).
+// The earlier phases' results for a sweep: y (forward) or z (backward); with
+// FP32 factors from f, y or the floats of z (Sys::zf).  A conversion from
+// FP64 costs the FP64 pipe what an FMA does: three per gathered block and
+// warp of a trio took a refactorisation and solve of 21,793 rows from 157.8
+// to 168.3 us.  (The launches per phase keep the conversions: there the
+// floats' stores cost as much, 3270 against 3247 us at 949,871 rows.)
 template <typename TF>
-__device__ __forceinline__ Vec3<TF> sweep_gather(const void *y, const double *z, bool fwd, int j) {
-  if (sizeof(TF) != sizeof(double) && fwd) return load3cg(static_cast<const TF *>(y) + 3ll * j);
-  const Vec3<double> v = load3cg((fwd ? static_cast<const double *>(y) : z) + 3ll * j);
-  return {(TF)v.c0, (TF)v.c1, (TF)v.c2};
+__device__ __forceinline__ Vec3<TF> sweep_gather(const void *y, const double *z, const float *f, bool fwd, int j) {
+  if constexpr (sizeof(TF) == 4) {
+    return load3cg(f + 3ll * j);
+  } else {
+    const Vec3<double> v = load3cg((fwd ? static_cast<const double *>(y) : z) + 3ll * j);
+    return {(TF)v.c0, (TF)v.c1, (TF)v.c2};
+  }
 }
 
 // One slice of a sweep over the phase's rows [E.z, E.w): fwd_rows (fwd; the
@@ -329,6 +337,7 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
   const int32_t *rp = fwd ? S.l_rp : S.u_rp, *col = fwd ? S.l_col : S.u_col;
   const TF *lu = static_cast<const TF *>(S.lu);
   const TF *vals = lu + (fwd ? 0 : S.u_off);
+  const float *zf = sizeof(TF) == 4 ? (fwd ? static_cast<const float *>(S.y) : S.zf) : nullptr;
   const int len = (i < S.n) ? __ldg(rp + i + 1) - __ldg(rp + i) : 0;
   int base = __ldg(rp + s0);
   const int maxlen = __reduce_max_sync(0xffffffffu, len);
@@ -370,11 +379,11 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
     if (u0) j0 = __ldcs(col + b0 + q0);
     if (u1) j1 = __ldcs(col + b1 + q1);
     if (u0) {
-      const Vec3<TF> v = sweep_gather<TF>(S.y, z, fwd, j0);
+      const Vec3<TF> v = sweep_gather<TF>(S.y, z, zf, fwd, j0);
       blk_sub<TF>(vals + 9ll * b0 + q0, __popc(m0), v.c0, v.c1, v.c2, a.c0, a.c1, a.c2);
     }
     if (u1) {
-      const Vec3<TF> v = sweep_gather<TF>(S.y, z, fwd, j1);
+      const Vec3<TF> v = sweep_gather<TF>(S.y, z, zf, fwd, j1);
       blk_sub<TF>(vals + 9ll * b1 + q1, __popc(m1), v.c0, v.c1, v.c2, a.c0, a.c1, a.c2);
     }
   }
@@ -389,7 +398,11 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
   if (!fwd || eager) {
     TF d[9];
     load_dinv<TF>(lu + S.d_off + (int64_t)kSliceVals * sl + lane, d);
-    store_dinv_product<TF>(z + 3ll * i, d, a.c0, a.c1, a.c2);
+    const Vec3<TF> v = store_dinv_product<TF>(z + 3ll * i, d, a.c0, a.c1, a.c2);
+    if constexpr (sizeof(TF) == 4) {
+      float *f = S.zf + 3ll * i;
+      f[0] = v.c0; f[1] = v.c1; f[2] = v.c2;
+    }
     if (kPlain) store_dinv_product<TF>(S.x_out + o, d, a.c0, a.c1, a.c2);
   }
   if (fwd && ((M.y >> lane) & 1u)) {
@@ -622,6 +635,7 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   const int32_t *rp = fwd ? S.l_rp : S.u_rp, *col = fwd ? S.l_col : S.u_col;
   const TF *lu = static_cast<const TF *>(S.lu);
   const TF *vals = lu + (fwd ? 0 : S.u_off);
+  const float *zf = sizeof(TF) == 4 ? (fwd ? static_cast<const float *>(S.y) : S.zf) : nullptr;
   const int len = (i < S.n) ? __ldg(rp + i + 1) - __ldg(rp + i) : 0;
   const int lead = act ? len : 0;
   int base = __ldg(rp + s0);
@@ -655,7 +669,7 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
 #pragma unroll
   for (int k = 0; k < kPre; ++k) {
     vv[k] = {TF(0), TF(0), TF(0)};
-    if (lead > k) vv[k] = sweep_gather<TF>(S.y, z, fwd, jp[k]);
+    if (lead > k) vv[k] = sweep_gather<TF>(S.y, z, zf, fwd, jp[k]);
   }
   const TF y0 = a;  // the backward sweep's y_i
   if (act && fwd && kPlain) {
@@ -675,7 +689,7 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
     const unsigned m = __ballot_sync(0xffffffffu, len > k);
     if (lead > k) {
       const int cnt = __popc(m), q = __popc(m & lt);
-      const Vec3<TF> v = sweep_gather<TF>(S.y, z, fwd, __ldcs(col + base + q));
+      const Vec3<TF> v = sweep_gather<TF>(S.y, z, zf, fwd, __ldcs(col + base + q));
       const TF *b = vals + 9ll * base + q + 3 * r * cnt;
       const TF b0 = __ldcs(b), b1 = __ldcs(b + cnt), b2 = __ldcs(b + 2 * cnt);
       a = fma(-b0, v.c0, fma(-b1, v.c1, fma(-b2, v.c2, a)));
@@ -691,8 +705,10 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   if (!kPlain && !fwd && sizeof(TF) == sizeof(double) && S.uz && ((__ldg(S.sp_mask + sl).y >> lane) & 1u))
     S.uz[e] = (double)(y0 - a);
   if (use_d) {
-    const double v = (double)fma(d[0], a0, fma(d[1], a1, d[2] * a2));
+    const TF f = fma(d[0], a0, fma(d[1], a1, d[2] * a2));
+    const double v = (double)f;
     z[e] = v;
+    if constexpr (sizeof(TF) == 4) S.zf[e] = f;
     if (kPlain) S.x_out[o] = v;
   }
   if (fwd && ((M.y >> lane) & 1u)) y[e] = a;

@@ -1200,6 +1200,7 @@ opm_status alloc_system(opm_solver *h, const Analysis &an) {
     float *lu, *y;
     if ((s = dalloc(A, bytes, st, &lu, (size_t)an.lu_vals)) != OPM_OK) return s;
     if ((s = dalloc(A, bytes, st, &y, 3 * (size_t)nb)) != OPM_OK) return s;
+    if ((s = dalloc(A, bytes, st, &S.zf, 3 * (size_t)nb)) != OPM_OK) return s;
     S.lu = lu;
     S.y = y;
   } else {

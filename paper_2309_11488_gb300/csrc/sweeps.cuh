@@ -128,10 +128,13 @@ __device__ __forceinline__ void load_dinv(const TF *D, TF (&d)[9]) {
 }
 
 template <typename TF>
-__device__ __forceinline__ void store_dinv_product(double *zi, const TF (&d)[9], TF a0, TF a1, TF a2) {
-  zi[0] = (double)fma(d[0], a0, fma(d[1], a1, d[2] * a2));
-  zi[1] = (double)fma(d[3], a0, fma(d[4], a1, d[5] * a2));
-  zi[2] = (double)fma(d[6], a0, fma(d[7], a1, d[8] * a2));
+__device__ __forceinline__ Vec3<TF> store_dinv_product(double *zi, const TF (&d)[9], TF a0, TF a1, TF a2) {
+  const Vec3<TF> v{fma(d[0], a0, fma(d[1], a1, d[2] * a2)), fma(d[3], a0, fma(d[4], a1, d[5] * a2)),
+                   fma(d[6], a0, fma(d[7], a1, d[8] * a2))};
+  zi[0] = (double)v.c0;
+  zi[1] = (double)v.c1;
+  zi[2] = (double)v.c2;
+  return v;
 }
 
 template <int MODE>
