@@ -304,6 +304,15 @@ constexpr int kMaxTriSweeps = 64;
 
 int blocks8(int entries) { return std::max(1, (entries + 7) / 8); }
 
+// Threads of a CTA of a large phase's launch (a slice per warp).  An SM takes
+// whole CTAs, and past a full round of them (four of 256 threads per SM) the
+// busiest SM of a phase of 949,871 rows worked 8% longer than the mean with
+// 256 threads.  Refactor + solve there, FP64 / FP32 factors: 256 threads 3505 /
+// 3265 us, 128 threads 3443 / 3219, 64 threads 3452 / 3225.  Within one round
+// 256 stay: GMRES at 249,053 rows takes 1604 us with them, 1622 with 128.
+int phase_threads(const Runner &R, int entries) { return entries > 32 * R.sms ? 128 : 256; }
+int phase_blocks(int entries, int threads) { return (entries + threads / 32 - 1) / (threads / 32); }
+
 // Iterative ILU0: the initial guess, then cp_sweeps synchronous sweeps,
 // alternating between the two factor buffers so that the last sweep writes
 // the one the solver reads (sweep t of T writes buffer (T - t) & 1).
@@ -331,8 +340,9 @@ int launch_factor_t(Runner &R, cudaStream_t st) {
   for (int c = 0; c < R.nphases; ++c) {
     const int cnt = R.fwd_ptr[c + 1] - R.fwd_ptr[c];
     if (cnt == 0) continue;
+    const int nt = phase_threads(R, cnt);
     if (cnt <= R.small_entries) launch_pdl(k_factor_phase<TF, kFp32, 1>, (cnt + 1) / 2, 64, st, R.B, c);
-    else launch_pdl(k_factor_phase<TF, true, 4, kFp32>, blocks8(cnt), 256, st, R.B, c);
+    else launch_pdl(k_factor_phase<TF, true, 4, kFp32>, phase_blocks(cnt, nt), nt, st, R.B, c);
     ++n;
   }
   return n;
@@ -352,12 +362,13 @@ constexpr int sweep_preload() {
 template <typename TF, int MODE, bool FWD>
 void launch_sweep_phase(Runner &R, cudaStream_t st, int c, int cnt) {
   constexpr int P = sweep_preload<TF>();
+  const int nt = phase_threads(R, cnt);
   if (cnt <= R.small_entries) {
     if (FWD) launch_pdl(k_fwd_phase<TF, MODE, P>, (cnt + 1) / 2, 64, st, R.B, c);
     else launch_pdl(k_bwd_phase<TF, MODE, P>, (cnt + 1) / 2, 64, st, R.B, c);
   } else {
-    if (FWD) launch_pdl(k_fwd_phase<TF, MODE, 0>, blocks8(cnt), 256, st, R.B, c);
-    else launch_pdl(k_bwd_phase<TF, MODE, 0>, blocks8(cnt), 256, st, R.B, c);
+    if (FWD) launch_pdl(k_fwd_phase<TF, MODE, 0>, phase_blocks(cnt, nt), nt, st, R.B, c);
+    else launch_pdl(k_bwd_phase<TF, MODE, 0>, phase_blocks(cnt, nt), nt, st, R.B, c);
   }
 }
 
@@ -387,7 +398,8 @@ int launch_apply_t(Runner &R, cudaStream_t st) {
   for (int c = 0; c < R.nphases; ++c) {
     const int cnt = R.fwd_ptr[c + 1] - R.fwd_ptr[c];
     if (cnt == 0) continue;
-    if (c == 0) launch_pdl(k_fwd_first<TF, MODE>, blocks8(cnt), 256, st, R.B);  // no L blocks in phase 0
+    const int nt = phase_threads(R, cnt);
+    if (c == 0) launch_pdl(k_fwd_first<TF, MODE>, phase_blocks(cnt, nt), nt, st, R.B);  // no L blocks in phase 0
     else launch_sweep_phase<TF, MODE, true>(R, st, c, cnt);
     ++n;
   }

@@ -285,7 +285,7 @@ __device__ __forceinline__ void bwd_rows(const Sys &S, int sl, int r0, int r1) {
 template <typename TF, int MODE>
 __global__ void __launch_bounds__(256, 8) k_fwd_first(Batch B) {
   pdl_trigger();
-  const int e = __ldg(B.fwd_ptr) + blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int e = __ldg(B.fwd_ptr) + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (e >= __ldg(B.fwd_ptr + 1)) return;
   const int4 E = B.ent[e];
   const Sys &S = B.sys[E.x];
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(256, 8) k_fwd_first(Batch B) {
 }
 
 // One launch per phase, one sweep entry (a 32-row slice) per warp.  PRE = 0:
-// throughput form for large phases (256 threads); PRE > 0: latency form for
+// throughput form for large phases (128 or 256 threads); PRE > 0: latency form for
 // small phases (64 threads, so the few warps spread over all SMs).
 template <typename TF, int MODE, int PRE>
 __global__ void __launch_bounds__(PRE > 0 ? 64 : 256, PRE > 0 ? 1 : 4) k_fwd_phase(Batch B, int c) {
