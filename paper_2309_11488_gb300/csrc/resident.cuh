@@ -594,6 +594,11 @@ __device__ __forceinline__ void vector_unit(ResCtx &c, int u, bool setup) {
 // hold, the first kPre blocks are loaded before the wait without spills.  A
 // component's chain of operations is that of the one-warp form.
 
+// The blocks and their columns are loaded with the default cache policy, not as
+// streams: a system of these sizes stays in L2 from one product to the next.
+// Evict-first loads took (us, refactor + solve) 252.4 against 249.7 at 44,431
+// rows, 449.4 against 433.0 at 60,793, 32.8 against 31.4 for an application
+// alone at 44,431.
 constexpr int kPre = 6;  // blocks loaded ahead: the couplings of a cell on a grid
 
 // The first kPre blocks of the lane's row, row r of each: columns and values.
@@ -611,10 +616,10 @@ __device__ __forceinline__ int preload_row(const int32_t *col, const T *vals, in
     if (lead > k) {
       const int q = __popc(m & lt), cnt = __popc(m);
       const T *v = vals + 9ll * base + q + 3 * r * cnt;
-      jp[k] = __ldcs(col + base + q);
-      bp[k][0] = __ldcs(v);
-      bp[k][1] = __ldcs(v + cnt);
-      bp[k][2] = __ldcs(v + 2 * cnt);
+      jp[k] = __ldca(col + base + q);
+      bp[k][0] = __ldca(v);
+      bp[k][1] = __ldca(v + cnt);
+      bp[k][2] = __ldca(v + 2 * cnt);
     }
     base += __popc(m);
   }
@@ -646,9 +651,9 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   base = preload_row<TF>(col, vals, len, lead, base, r, jp, bp);
   if (use_d) {
     const TF *D = lu + S.d_off + (int64_t)kSliceVals * sl + lane + 96 * r;
-    d[0] = __ldcs(D);
-    d[1] = __ldcs(D + 32);
-    d[2] = __ldcs(D + 64);
+    d[0] = __ldca(D);
+    d[1] = __ldca(D + 32);
+    d[2] = __ldca(D + 64);
   }
   if (FIRST) c.wait();
   double h = 0.0, vo = 0.0, po = 0.0;
@@ -689,9 +694,9 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
     const unsigned m = __ballot_sync(0xffffffffu, len > k);
     if (lead > k) {
       const int cnt = __popc(m), q = __popc(m & lt);
-      const Vec3<TF> v = sweep_gather<TF>(S.y, z, zf, fwd, __ldcs(col + base + q));
+      const Vec3<TF> v = sweep_gather<TF>(S.y, z, zf, fwd, __ldca(col + base + q));
       const TF *b = vals + 9ll * base + q + 3 * r * cnt;
-      const TF b0 = __ldcs(b), b1 = __ldcs(b + cnt), b2 = __ldcs(b + 2 * cnt);
+      const TF b0 = __ldca(b), b1 = __ldca(b + cnt), b2 = __ldca(b + 2 * cnt);
       a = fma(-b0, v.c0, fma(-b1, v.c1, fma(-b2, v.c2, a)));
     }
     base += __popc(m);
@@ -758,9 +763,9 @@ __device__ __forceinline__ void product_trio(ResCtx &c, int4 E, int step, bool r
     const unsigned m = __ballot_sync(0xffffffffu, len > k);
     if (lead > k) {
       const int cnt = __popc(m), p = __popc(m & lt);
-      const Vec3<double> x = load3cg(io.x + 3ll * __ldcs(S.a_col + base + p));
+      const Vec3<double> x = load3cg(io.x + 3ll * __ldca(S.a_col + base + p));
       const double *b = S.a_val + 9ll * base + p + 3 * r * cnt;
-      const double b0 = __ldcs(b), b1 = __ldcs(b + cnt), b2 = __ldcs(b + 2 * cnt);
+      const double b0 = __ldca(b), b1 = __ldca(b + cnt), b2 = __ldca(b + 2 * cnt);
       y = fma(b0, x.c0, fma(b1, x.c1, fma(b2, x.c2, y)));
     }
     base += __popc(m);
