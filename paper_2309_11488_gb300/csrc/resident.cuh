@@ -81,6 +81,8 @@ struct ResShared {
   Sys sys[kResMaxSys];
   Scal sc[kResMaxSys];
   int dead, last;
+  int32_t phase0;                           // entries of the first forward phase
+  int4 first[kResidentThreads / 32];        // the warps' first entry of it
   double ex[kTrios][2][4][3][32];  // a trio's exchange: two units in turn, up to four rows per lane
 };
 
@@ -1019,10 +1021,12 @@ __device__ __forceinline__ void resident_factor(ResCtx &c) {
 template <typename TF, int MODE, bool TRIO>
 __device__ __forceinline__ void resident_apply(ResCtx &c, bool second) {
   const Batch &B = c.R.B;
-  // the first phase's rows have no L blocks: nothing to load ahead
+  // The first phase's rows have no L blocks, so there is nothing to load ahead
+  // of the wait but the warp's entry, which is kept: finding it again took two
+  // loads from L2, one after the other.
 #pragma unroll 1
-  for (int e = __ldg(B.fwd_ptr) + c.g, e1 = __ldg(B.fwd_ptr + 1); e < e1; e += c.W) {
-    const int4 E = __ldg(B.ent + e);
+  for (int e = c.g, e1 = c.sm.phase0; e < e1; e += c.W) {
+    const int4 E = e == c.g ? c.sm.first[c.wp] : __ldg(B.ent + e);
     if (!c.runs(E.x)) continue;
     if constexpr (TRIO) sweep_trio<TF, MODE, false>(c, E, true, second);
     else sweep_unit<TF, MODE>(c, E, true, second);
@@ -1064,6 +1068,9 @@ __device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &s
     c.g = c.warp_id();  // consecutive units go to different SMs
     c.W = c.warps();
   }
+  const int phase0 = __ldg(B.fwd_ptr + 1);
+  if (threadIdx.x == 0) sm.phase0 = phase0;
+  if (c.lane == 0 && c.g < phase0) sm.first[wp] = __ldg(B.ent + c.g);
   const int4 *src = reinterpret_cast<const int4 *>(B.nsys == 1 ? &R.one : B.sys);
   int4 *dst = reinterpret_cast<int4 *>(sm.sys);
   static_assert(sizeof(Sys) % sizeof(int4) == 0, "descriptors are copied in 16-byte pieces");
