@@ -587,10 +587,12 @@ opm_status opm_autotune_batch(int32_t nsys, const int32_t *nb, const int32_t *co
  * Its scratch is a fixed 131,328-byte array in device memory that every GPU
  * using the library holds until the process exits.  The first call on a
  * device looks up that array's device address (once per device, with the
- * device current) and keeps it.  Calls after a cudaDeviceReset of that
- * device are not supported.
- * All calls share the array: calls that overlap on the GPU race and must be
- * serialised by the caller.
+ * device current) and keeps it.  The first call also registers 64 KB of the
+ * library's own static host memory with CUDA (cudaHostRegister; kept until
+ * the process exits), through which the outcome comes back: one word per
+ * device.  Calls after a cudaDeviceReset of that device are not supported.
+ * All calls on one GPU share the array: calls that overlap on it race and
+ * must be serialised by the caller.  Calls on different GPUs are independent.
  */
 opm_status opm_bsr_residual_noalloc(int32_t nb, const int32_t *rowptr, const int32_t *colidx,
                                     const double *vals, const double *x, const double *b, double *r,

@@ -14,11 +14,12 @@
 // library holds these 131,328 bytes until the process exits, every call
 // shares them, and they keep the last call's partial sums.  The counter and
 // the error word are zero between calls (the last CTA of a call clears them).
-// The outcome reaches the host through a word of the library's own static
-// memory, which the first call registers with CUDA (cudaHostRegister): a
-// copy back into pageable memory took longer than a small residual.  Calls
-// that overlap on the GPU (on two streams, or from two host threads) race on
-// the array and give wrong results: serialise them.
+// The outcome reaches the host through the device's word in the library's own
+// static memory, which the first call registers with CUDA (cudaHostRegister):
+// a copy back into pageable memory took longer than a small residual.  Calls
+// that overlap on one GPU (on two streams, or from two host threads) race on
+// the array and give wrong results: serialise them.  Calls on different GPUs
+// share nothing.
 //
 // The caller's pattern is not validated on the host (that would need a copy
 // of it).  The kernel checks what it can before each access: a row whose
@@ -35,8 +36,11 @@
 #include <mutex>
 
 #include "../../include/opm_bsr.h"
+#include "noalloc_calls.h"
 
 namespace {
+
+using opm::kNoallocDevices;
 
 constexpr int kNaMaxRows = 2097152;
 constexpr int kNaMaxTiles = 8192;              // CTAs of a call
@@ -50,20 +54,15 @@ constexpr size_t kNaScratchBytes = kNaCounterBytes + sizeof(double) * 2 * kNaMax
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaScratchBytes];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
-unsigned char *g_scratch_ptr[kMaxDevices] = {};
+unsigned char *g_scratch_ptr[kNoallocDevices] = {};
 
-// Device address of the scratch array for the current device (looked up once
+// Device address of the scratch array for the current device dev (looked up once
 // per device, with that device current, and kept: calls after a
 // cudaDeviceReset of that device are not supported, since the reloaded
 // module may place the array elsewhere).
-opm_status scratch_address(unsigned char **out) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-    cudaGetLastError();
-    return OPM_ERR_CUDA;
-  }
+opm_status scratch_address(int dev, unsigned char **out) {
+  if (dev < 0 || dev >= kNoallocDevices) return OPM_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   if (!g_scratch_ptr[dev]) {
     void *p = nullptr;
@@ -257,28 +256,27 @@ __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
   *outcome = faulty ? 2u : 1u;
 }
 
-// The word through which a call's outcome reaches the host: in a page of the
-// library's own, registered once for all devices.
-constexpr size_t kHostPage = 65536;
-alignas(kHostPage) unsigned char g_host_page[kHostPage];
+opm::NoallocPage g_host_page;
 bool g_host_registered = false;
 
-// Its address on the current device, NULL when it cannot be registered.
-unsigned int *outcome_address() {
+// The address on the current device dev of its outcome word, NULL when the
+// page cannot be registered.
+unsigned int *outcome_address(int dev) {
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   if (!g_host_registered) {
-    if (cudaHostRegister(g_host_page, kHostPage, cudaHostRegisterPortable | cudaHostRegisterMapped) != cudaSuccess) {
+    if (cudaHostRegister(&g_host_page, sizeof(g_host_page), cudaHostRegisterPortable | cudaHostRegisterMapped) !=
+        cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
     g_host_registered = true;
   }
   void *p = nullptr;
-  if (cudaHostGetDevicePointer(&p, g_host_page, 0) != cudaSuccess) {
+  if (cudaHostGetDevicePointer(&p, &g_host_page, 0) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  return static_cast<unsigned int *>(p);
+  return const_cast<unsigned int *>(&static_cast<opm::NoallocPage *>(p)->line[dev].outcome);
 }
 
 }  // namespace
@@ -306,7 +304,7 @@ extern "C" opm_status opm_bsr_residual_noalloc(int32_t nb, const int32_t *rowptr
       !on_device(b, dev) || !on_device(r, dev))
     return OPM_ERR_ARG;
   unsigned char *scratch = nullptr;
-  opm_status s = scratch_address(&scratch);
+  opm_status s = scratch_address(dev, &scratch);
   if (s != OPM_OK) return s;
   // as many CTAs as fit on the device at once: a CTA's sums end in 20 FP64
   // additions per warp, as much as the product of one group
@@ -316,9 +314,9 @@ extern "C" opm_status opm_bsr_residual_noalloc(int32_t nb, const int32_t *rowptr
     return OPM_ERR_CUDA;
   }
   const int tiles = std::min((nb + kNaTile - 1) / kNaTile, std::min(8 * sms, kNaMaxTiles));
-  unsigned int *outcome = outcome_address();
+  unsigned int *outcome = outcome_address(dev);
   if (!outcome) return OPM_ERR_CUDA;
-  volatile unsigned int *word = reinterpret_cast<unsigned int *>(g_host_page);
+  volatile unsigned int *word = &g_host_page.line[dev].outcome;
   *word = 0u;
   k_residual_noalloc<<<tiles, kNaThreads, 0, st>>>(nb, rowptr, colidx, vals, x, b, r, norms, scratch, outcome);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess || *word == 0u) {
