@@ -306,7 +306,8 @@ void opm_analysis_destroy(opm_analysis a);
  *   stream; uses (m + 1) extra vectors of device memory, kept for later
  *   calls.  Not available on batches.
  * Returns OPM_OK, OPM_NOT_CONVERGED, OPM_ERR_ARG, OPM_ERR_ZERO_PIVOT (no
- * valid factors), OPM_ERR_BREAKDOWN (a zero rotation), OPM_ERR_NONFINITE,
+ * valid factors), OPM_ERR_TIMEOUT (the last refactorisation's wait expired:
+ * factor again), OPM_ERR_BREAKDOWN (a zero rotation), OPM_ERR_NONFINITE,
  * OPM_ERR_OOM or OPM_ERR_CUDA; on negative codes x is zero-filled.
  */
 opm_status opm_gmres_solve(opm_handle h, const double *b, double *x, double rtol, int32_t maxit,
@@ -364,7 +365,8 @@ opm_status opm_bicgstab_solve(opm_handle h, const double *b, double *x, double r
 opm_status opm_spmv(opm_handle h, const double *x, double *y);
 
 /* z = U^-1 L^-1 r with the current factors (Algorithm 1, equations 3-4);
- * r, z host or device, 3*nb doubles, caller's order. */
+ * r, z host or device, 3*nb doubles, caller's order.  OPM_ERR_TIMEOUT when a
+ * wait expired, here or in the refactorisation that left the factors. */
 opm_status opm_ilu_apply(opm_handle h, const double *r, double *z);
 
 /* Release the handle and all its device memory.  NULL is ignored.

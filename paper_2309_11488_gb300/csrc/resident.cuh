@@ -1090,7 +1090,9 @@ __device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &s
   return c;
 }
 
-// The end: the last CTA to leave writes the outcome and clears the device words.
+// The end: the last CTA to leave writes the outcome and clears the device
+// words.  After an expired wait no stage has written x: it zeroes it, as the
+// finish stage does for every other failure.
 __device__ __forceinline__ void resident_leave(ResCtx &c) {
   const Resident &R = c.R;
   ResShared &sm = c.sm;
@@ -1104,6 +1106,10 @@ __device__ __forceinline__ void resident_leave(ResCtx &c) {
   __syncthreads();
   if (!sm.last) return;
   const bool aborted = ld_acquire(&R.ctl->abort) != 0u;
+  if (aborted && solve)
+    for (int s = 0; s < R.B.nsys; ++s)
+      for (int64_t e = threadIdx.x; !sm.sys[s].skip && e < 3ll * sm.sys[s].n; e += blockDim.x)
+        sm.sys[s].x_out[e] = 0.0;
   for (int s = threadIdx.x; s < R.B.nsys; s += blockDim.x) {
     const Sys &S = sm.sys[s];
     const Scal &sc = sm.sc[s];

@@ -61,10 +61,12 @@ struct opm_solver {
   double *vec_in = nullptr, *vec_out = nullptr;  // caller-order staging
   int32_t last_err_row = -1;
   bool factors_ok = false;
+  bool factors_cut = false;      // the last refactorisation's wait expired: its factors are half built
   opm_timing timing{};
   cudaEvent_t ev[2] = {};
   opm::Runner *run = nullptr;    // batch of one
   bool async_pending = false;
+  bool async_factor = false;     // the pending launch refactors
 };
 
 struct opm_analysis_s {
@@ -76,6 +78,7 @@ struct opm_batch_s {
   std::vector<opm_solver *> members;
   std::vector<char> sat_out;  // members that sit the pending launch out
   bool async_pending = false;
+  bool async_factor = false;  // the pending launch refactors
 };
 
 namespace opm {
@@ -1121,6 +1124,7 @@ opm_status staged_vec(opm_solver *h, const double *src, const double **dev) {
 
 opm_status factor_impl(opm_solver *h, const double *vals) {
   h->factors_ok = false;
+  h->factors_cut = false;
   h->last_err_row = -1;
   if (h->n == 0) {
     h->factors_ok = true;
@@ -1518,6 +1522,7 @@ opm_status opm_gmres_solve(opm_handle h, const double *b, double *x, double rtol
   if (relres) *relres = 0.0;
   if (h->n == 0) return OPM_OK;
   if (!h->factors_ok) return OPM_ERR_ZERO_PIVOT;
+  if (h->factors_cut) return OPM_ERR_TIMEOUT;
   const int m = restart > 0 ? restart : 30;
   bool x_dev = false;
   opm_status s = prepare_solve(h, b, x, rtol, maxit, &x_dev);
@@ -1936,6 +1941,7 @@ opm_status opm_solve_launch(opm_handle h, const double *vals, const double *b, d
     CK(cudaEventRecord(R.ev_done, h->stream));  // completion now includes the copy back
   }
   h->async_pending = true;
+  h->async_factor = vals != nullptr;
   h->timing.launches += vals ? h->run->factor_launches : 0;
   return OPM_OK;
 }
@@ -1962,6 +1968,7 @@ opm_status opm_solve_wait(opm_handle h, int32_t *iters, double *relres) {
   } else {
     h->factors_ok = true;
   }
+  if (h->async_factor) h->factors_cut = r.status == OPM_ERR_TIMEOUT;
   if (iters) *iters = r.iters;
   if (relres) *relres = r.relres;
   return (opm_status)r.status;
@@ -2002,6 +2009,7 @@ opm_status opm_ilu_apply(opm_handle h, const double *r, double *z) {
   if (!h || (h->n > 0 && (!r || !z)) || h->async_pending) return OPM_ERR_ARG;
   if (h->n == 0) return OPM_OK;
   if (!h->factors_ok) return OPM_ERR_ZERO_PIVOT;
+  if (h->factors_cut) return OPM_ERR_TIMEOUT;
   const double *dr = nullptr;
   opm_status s = staged_vec(h, r, &dr);
   if (s != OPM_OK) return s;
@@ -2169,6 +2177,7 @@ opm_status opm_batch_factor(opm_batch b, const double *const *vals, opm_status *
   for (int i = 0; i < R.nsys; ++i) {
     opm_solver *h = b->members[i];
     const Result &r = R.h_res[i];
+    h->factors_cut = false;
     if (r.status < 0) {
       h->factors_ok = false;
       h->last_err_row = (r.err_row >= 0 && r.err_row < h->n) ? h->an.perm[r.err_row] : -1;
@@ -2251,6 +2260,7 @@ opm_status opm_batch_launch(opm_batch b, const double *const *vals, const double
   }
   if (s != OPM_OK) return s;
   b->async_pending = true;
+  b->async_factor = vals != nullptr;
   return OPM_OK;
 }
 
@@ -2279,6 +2289,7 @@ opm_status opm_batch_wait(opm_batch b, int32_t *iters, double *relres, opm_statu
     }
     const Result &r = R.h_res[i];
     h->factors_ok = r.status != OPM_ERR_ZERO_PIVOT;
+    if (b->async_factor) h->factors_cut = r.status == OPM_ERR_TIMEOUT;
     if (iters) iters[i] = r.iters;
     if (relres) relres[i] = r.relres;
     if (st) st[i] = (opm_status)r.status;
