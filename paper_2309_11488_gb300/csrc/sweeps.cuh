@@ -76,9 +76,7 @@ __device__ __forceinline__ void row_sub(const int32_t *__restrict__ col, const T
 }
 
 // The first PRE slabs of the lane's row, loaded ahead: column, block values.
-// Returns the first block of slab PRE.  Slabs that the row has not are zero:
-// left undefined, the arrays of a sweep inside a loop would count as carried
-// from one round to the next and be spilled (3.4 KB per thread).
+// Returns the first block of slab PRE.
 template <typename TF, int PRE>
 __device__ __forceinline__ int preload_slabs(const int32_t *__restrict__ col, const TF *__restrict__ vals, int len,
                                              int base, bool act, int (&jp)[PRE], TF (&bp)[PRE][9]) {
@@ -86,9 +84,6 @@ __device__ __forceinline__ int preload_slabs(const int32_t *__restrict__ col, co
 #pragma unroll
   for (int k = 0; k < PRE; ++k) {
     const unsigned m = __ballot_sync(0xffffffffu, len > k);
-    jp[k] = 0;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) bp[k][e] = TF(0);
     if (act && len > k) {
       const int q = __popc(m & lt), cnt = __popc(m);
       jp[k] = __ldcs(col + base + q);
@@ -105,10 +100,8 @@ template <typename TV, int PRE>
 __device__ __forceinline__ void gather_preloaded(const TV *vec, int len, bool act, const int (&jp)[PRE],
                                                  Vec3<TV> (&vv)[PRE]) {
 #pragma unroll
-  for (int k = 0; k < PRE; ++k) {
-    vv[k] = {TV(0), TV(0), TV(0)};
+  for (int k = 0; k < PRE; ++k)
     if (act && len > k) vv[k] = load3cg(vec + 3ll * jp[k]);
-  }
 }
 
 // a -= B_k v_k over the preloaded slabs, in slab order.
