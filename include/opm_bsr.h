@@ -593,8 +593,9 @@ opm_status opm_autotune_batch(int32_t nsys, const int32_t *nb, const int32_t *co
  * library's own static host memory with CUDA (cudaHostRegister; kept until
  * the process exits), through which the outcome comes back: one word per
  * device.  Calls after a cudaDeviceReset of that device are not supported.
- * All calls on one GPU share the array: calls that overlap on it race and
- * must be serialised by the caller.  Calls on different GPUs are independent.
+ * All calls on one GPU share the array: calls that overlap on it race (wrong
+ * norms or OPM_ERR_CUDA for those calls) and must be serialised by the caller.
+ * Calls on different GPUs are independent.
  */
 opm_status opm_bsr_residual_noalloc(int32_t nb, const int32_t *rowptr, const int32_t *colidx,
                                     const double *vals, const double *x, const double *b, double *r,

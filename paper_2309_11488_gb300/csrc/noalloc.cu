@@ -9,11 +9,12 @@
 // ||r||_2, ||b||_2 on the caller's own BSR arrays without creating a handle
 // and without allocating anything.
 //
-// Its only scratch (one partial sum pair per CTA, the last-CTA counter and a
-// pattern-error word) is the file-scope array below: every GPU that loads the
-// library holds these 131,328 bytes until the process exits, every call
-// shares them, and they keep the last call's partial sums.  The counter and
-// the error word are zero between calls (the last CTA of a call clears them).
+// Its only scratch (one partial sum pair per CTA, the CTAs' ticket counter and
+// a pattern-error word) is the file-scope array below: every GPU that loads
+// the library holds these 131,328 bytes until the process exits, every call
+// shares them, and they keep the last call's partial sums.  The counter runs
+// on from call to call and the error word holds the tag of the call that set
+// it, so no call depends on how an earlier one ended (noalloc_calls.h).
 // The outcome reaches the host through the device's word in the library's own
 // static memory, which the first call registers with CUDA (cudaHostRegister):
 // a copy back into pageable memory took longer than a small residual.  Calls
@@ -41,6 +42,8 @@
 namespace {
 
 using opm::kNoallocDevices;
+using opm::NoallocCall;
+using opm::NoallocLine;
 
 constexpr int kNaMaxRows = 2097152;
 constexpr int kNaMaxTiles = 8192;              // CTAs of a call
@@ -56,6 +59,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaScratchBytes
 
 std::mutex g_setup_mutex;
 unsigned char *g_scratch_ptr[kNoallocDevices] = {};
+opm::NoallocCalls g_calls[kNoallocDevices];
 
 // Device address of the scratch array for the current device dev (looked up once
 // per device, with that device current, and kept: calls after a
@@ -96,7 +100,8 @@ __device__ __forceinline__ void copy8_async(double *dst, const double *src) {
 // r = b - A x on the caller's BSR matrix (row-major 3x3 blocks); per-CTA
 // partials of ||r||^2 and ||b||^2 in the scratch array, summed by the last
 // CTA.  Pattern faults that can be seen from the row (see the file header)
-// skip the access and set the error word; the last CTA then writes NaN norms.
+// skip the access and set the error word to the call's tag; the last CTA then
+// writes NaN norms.
 //
 // A warp takes groups of kNaGroup rows, three lanes per row, one component
 // each (30 of 32 lanes at work on the FP64 pipe, which bounds the product:
@@ -113,7 +118,8 @@ __device__ __forceinline__ void copy8_async(double *dst, const double *src) {
 __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
     int32_t nb, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
     const double *__restrict__ vals, const double *__restrict__ x, const double *__restrict__ b,
-    double *__restrict__ r, double *__restrict__ norms, unsigned char *scratch, volatile unsigned int *outcome) {
+    double *__restrict__ r, double *__restrict__ norms, unsigned char *scratch, NoallocLine *line, uint32_t base,
+    uint32_t tag) {
   __shared__ double sv[kNaWarps][9 * kNaChunk];
   __shared__ double sx[kNaWarps][3 * kNaChunk];
   __shared__ double sm[2][kNaWarps];
@@ -202,7 +208,7 @@ __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
       bb = fma(bi, bi, bb);
     }
   }
-  if (fault) atomicOr(bad, 1u);
+  if (fault) atomicExch(bad, tag);
   for (int o = 16; o > 0; o >>= 1) {
     rr += __shfl_xor_sync(all, rr, o);
     bb += __shfl_xor_sync(all, bb, o);
@@ -221,7 +227,9 @@ __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
     partials[2 * blockIdx.x] = s0;
     partials[2 * blockIdx.x + 1] = s1;
     __threadfence();
-    amlast = atomicAdd(counter, 1u) == gridDim.x - 1;
+    const uint32_t ticket = atomicAdd(counter, 1u);
+    amlast = opm::noalloc_is_last(ticket, base, gridDim.x);
+    if (opm::noalloc_is_foreign(ticket, base, gridDim.x)) line->spoilt = tag;
   }
   __syncthreads();
   if (!amlast) return;
@@ -248,20 +256,18 @@ __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
     s0 += sm[0][w];
     s1 += sm[1][w];
   }
-  const bool faulty = __ldcg(bad) != 0u;
+  const bool faulty = __ldcg(bad) == tag;
   norms[0] = faulty ? nan("") : sqrt(s0);
   norms[1] = faulty ? nan("") : sqrt(s1);
-  *counter = 0;
-  *bad = 0;
-  *outcome = faulty ? 2u : 1u;
+  line->outcome = opm::noalloc_outcome(tag, faulty ? opm::kNoallocFault : opm::kNoallocDone);
 }
 
 opm::NoallocPage g_host_page;
 bool g_host_registered = false;
 
-// The address on the current device dev of its outcome word, NULL when the
-// page cannot be registered.
-unsigned int *outcome_address(int dev) {
+// The address on the current device dev of its line, NULL when the page
+// cannot be registered.
+NoallocLine *line_address(int dev) {
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   if (!g_host_registered) {
     if (cudaHostRegister(&g_host_page, sizeof(g_host_page), cudaHostRegisterPortable | cudaHostRegisterMapped) !=
@@ -276,7 +282,7 @@ unsigned int *outcome_address(int dev) {
     cudaGetLastError();
     return nullptr;
   }
-  return const_cast<unsigned int *>(&static_cast<opm::NoallocPage *>(p)->line[dev].outcome);
+  return &static_cast<opm::NoallocPage *>(p)->line[dev];
 }
 
 }  // namespace
@@ -314,14 +320,27 @@ extern "C" opm_status opm_bsr_residual_noalloc(int32_t nb, const int32_t *rowptr
     return OPM_ERR_CUDA;
   }
   const int tiles = std::min((nb + kNaTile - 1) / kNaTile, std::min(8 * sms, kNaMaxTiles));
-  unsigned int *outcome = outcome_address(dev);
-  if (!outcome) return OPM_ERR_CUDA;
-  volatile unsigned int *word = &g_host_page.line[dev].outcome;
-  *word = 0u;
-  k_residual_noalloc<<<tiles, kNaThreads, 0, st>>>(nb, rowptr, colidx, vals, x, b, r, norms, scratch, outcome);
-  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess || *word == 0u) {
+  NoallocLine *line = line_address(dev);
+  if (!line) return OPM_ERR_CUDA;
+  NoallocCall call;
+  {
+    std::lock_guard<std::mutex> lock(g_setup_mutex);
+    call = g_calls[dev].begin((uint32_t)tiles);
+  }
+  bool ran = !call.clear || cudaMemsetAsync(scratch, 0, kNaCounterBytes, st) == cudaSuccess;
+  if (ran) {
+    k_residual_noalloc<<<tiles, kNaThreads, 0, st>>>(nb, rowptr, colidx, vals, x, b, r, norms, scratch, line,
+                                                     call.base, call.tag);
+    ran = cudaGetLastError() == cudaSuccess;
+    ran = cudaStreamSynchronize(st) == cudaSuccess && ran;
+  }
+  const NoallocLine &out = g_host_page.line[dev];
+  const uint64_t outcome = out.outcome;
+  if (!ran || out.spoilt == call.tag || outcome >> 32 != call.tag) {
     cudaGetLastError();
+    std::lock_guard<std::mutex> lock(g_setup_mutex);
+    g_calls[dev].unsure = true;
     return OPM_ERR_CUDA;
   }
-  return *word == 2u ? OPM_ERR_PATTERN : OPM_OK;
+  return (uint32_t)outcome == opm::kNoallocFault ? OPM_ERR_PATTERN : OPM_OK;
 }
