@@ -120,7 +120,10 @@ typedef struct opm_options {
                             solve loop (the loop condition is tested after
                             each body); 0 = default (2)                      */
   int32_t spin_limit_us; /* bound of every device-side wait in microseconds;
-                            0 = default (2,000,000)                           */
+                            0 = default (2,000,000).  The launch of a single
+                            system under OPM_SWEEP_AUTO waits at least
+                            100,000, not counting time in which the context
+                            was switched out                                 */
   int32_t debug_skip_item; /* test hook, -1 = off: the CTA with this index
                             never arrives at the grid barriers of the
                             cooperative launches, so the other CTAs'

@@ -94,6 +94,7 @@ struct Analysis {
   int64_t d_off = 0;                          // first value of Dinv inside the factor values
   int64_t lu_vals = 0;                        // total factor values
   int32_t max_row_len = 0;
+  int64_t max_chain = 0;                      // longest row's blocks, or elimination steps (its L blocks and updates)
 };
 
 // Validates and analyses the pattern; returns OPM_OK or a pattern error with

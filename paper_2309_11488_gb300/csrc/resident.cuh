@@ -71,6 +71,10 @@ struct Scal {
   int32_t status, k, iters, maxit, half, pad;
 };
 
+// Between two looks at the clock a wait counts at most this long: a context
+// that was switched out (a time slice, a debugger) has not waited.
+constexpr uint64_t kPollGapNs = 1000000;
+
 constexpr int kResMaxSys = 16;  // systems of one launch (descriptors and scalars in shared memory)
 
 constexpr int kTrios = 5;       // trios of a CTA of the trio form
@@ -197,11 +201,14 @@ struct ResCtx {
     if (boss) {
       bool d = dead || (int)blockIdx.x == R.B.skip_cta;
       if (!d) {
-        const uint64_t t0 = gtimer();
+        uint64_t last = gtimer(), waited = 0;
         for (uint32_t it = 1; (int32_t)(ld_acquire(&R.ctl->arrive) - target) < 0; ++it) {
           if ((it & 63u) == 0u) {
+            const uint64_t now = gtimer(), gap = now - last;
+            last = now;
+            waited += gap < kPollGapNs ? gap : kPollGapNs;
             if (ld_acquire(&R.ctl->abort) != 0u) d = true;
-            else if (gtimer() - t0 > R.B.spin_limit_ns) {
+            else if (waited > R.B.spin_limit_ns) {
               atomicExch(&R.ctl->abort, 1u);
               d = true;
             }

@@ -678,6 +678,13 @@ uint64_t spin_ns(const opm_options &o) {
   return (uint64_t)(o.spin_limit_us > 0 ? o.spin_limit_us : 2000000) * 1000ull;
 }
 
+// Bounds that keep a resident launch from running out of time over its own
+// work, which the launches per phase have no limit for: a wait lasts at least
+// kResidentWaitNs, and no lane of a stage takes more than kResidentChain
+// dependent steps of one to two microseconds (opm::Analysis::max_chain).
+constexpr uint64_t kResidentWaitNs = 100000000;
+constexpr int64_t kResidentChain = 8192;
+
 int chunk_of(const opm_options &o) { return o.chunk > 0 ? o.chunk : 2; }
 
 template <typename TF>
@@ -692,6 +699,7 @@ const void *resident_kernel(bool trio, bool apply) {
 opm_status resident_create(Runner &R, int max_entries) {
   if (R.nsys > 1 || R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(R.nall, R.sms)) return OPM_OK;
   if (R.stream && !shares_device(R.nall, R.sms)) return OPM_OK;
+  if (R.mem[0]->an.max_chain > kResidentChain) return OPM_OK;
   const bool trio = resident_trios(R.nall, R.sms);
   R.res_kernel = R.fp32 ? resident_kernel<float>(trio, false) : resident_kernel<double>(trio, false);
   R.res_apply = R.fp32 ? resident_kernel<float>(trio, true) : resident_kernel<double>(trio, true);
@@ -767,6 +775,7 @@ opm_status resident_create(Runner &R, int max_entries) {
   CK(cudaMemsetAsync(A.err, 0, sizeof(int32_t) * 2 * R.nsys, R.stream));
   CK(cudaMemsetAsync(A.ctl, 0, sizeof(ResidentCtl), R.stream));
   A.B = R.B;
+  A.B.spin_limit_ns = std::max(R.B.spin_limit_ns, kResidentWaitNs);
   A.ds = {sum_s, d_os, d_gs, d_gos, (int)grp_s.size(), off_s.back()};
   A.du = {sum_u, d_ou, d_gu, d_gou, (int)grp_u.size(), off_u.back()};
   A.nupd = 8 * R.ntiles;
@@ -1284,6 +1293,7 @@ void copy_host_part(Analysis &dst, const Analysis &src) {
   dst.d_off = src.d_off;
   dst.lu_vals = src.lu_vals;
   dst.max_row_len = src.max_row_len;
+  dst.max_chain = src.max_chain;
   dst.nnzb_product = src.nnzb_product;
   dst.rows_identity = src.rows_identity;
   dst.rows_reuse = src.rows_reuse;

@@ -528,6 +528,11 @@ opm_status analyse(int32_t n, const int32_t *rowptr, const int32_t *colidx, cons
   }
   if (an.upd_dst.size() >= ((size_t)1 << 31)) return OPM_ERR_ARG;
   an.nupd = (int64_t)an.upd_dst.size();
+  an.max_chain = an.max_row_len;
+  for (int32_t ni = 0; ni < n; ++ni) {
+    const int32_t l0 = an.l_rowptr[ni], l1 = an.l_rowptr[ni + 1];
+    an.max_chain = std::max<int64_t>(an.max_chain, (int64_t)(l1 - l0) + an.upd_ptr[l1] - an.upd_ptr[l0]);
+  }
 
   // ---- what the products after an application walk (sp_mask, sp_len)
   an.sp_mask.assign((size_t)(2 * nslices), 0u);

@@ -60,3 +60,39 @@ def test_expired_wait_zeroes_x_and_leaves_no_factors(n, precision):
         assert sv.factor(vals) == opm.OPM_OK
         got = sv.solve(b, rtol=1e-4)
         assert got[1:] == want[1:] and torch.equal(got[0], want[0]) and torch.equal(sv.ilu_apply(b), z)
+
+
+def hub_system(n):
+    """n - 1 rows coupled to the last one alone: in natural order two phases, the second a single long row."""
+    i = np.arange(n - 1, dtype=np.int32)
+    rowptr = np.concatenate([2 * np.arange(n, dtype=np.int32), [2 * (n - 1) + n]]).astype(np.int32)
+    colidx = np.concatenate([np.stack([i, np.full_like(i, n - 1)], 1).ravel(), np.arange(n, dtype=np.int32)])
+    rng = np.random.default_rng(n)
+    vals = rng.uniform(-1e-3, 1e-3, (len(colidx), 9))
+    rows = np.repeat(np.arange(n), np.diff(rowptr))
+    vals[rows == colidx] += 10.0 * np.eye(3).ravel()
+    vals[-1] += 1e-2 * n * np.eye(3).ravel()
+    return rowptr, colidx, vals
+
+
+@pytest.mark.parametrize("case", ["long_row", "short_limit"])
+def test_own_work_is_no_timeout(case):
+    """A limit shorter than a stage's own work: the launches per phase have none, and AUTO takes neither a row of
+    tens of thousands of dependent steps nor a limit of a microsecond for an expired wait."""
+    if case == "long_row":
+        rp, ci, vals = hub_system(20_000)
+    else:
+        s = synth.config2()
+        rp, ci, vals = s.rowptr, s.colidx, s.vals
+    nb = len(rp) - 1
+    b = torch.ones(3 * nb, dtype=torch.float64, device="cuda")
+    got = []
+    for sweep, limit in (("per_phase", 0), ("auto", 1 if case == "short_limit" else 1000)):
+        o = opm.opm_options_default(sweep_launch=sweep, spin_limit_us=limit,
+                                    schedule="natural" if case == "long_row" else "auto")
+        st, h = opm.opm_bsr_create(nb, rp, ci, vals, o, check=False)
+        assert st == opm.OPM_OK
+        x = torch.empty_like(b)
+        got.append((opm.opm_bicgstab_solve(h, b, x, rtol=1e-6), x))
+        opm.opm_destroy(h)
+    assert got[0][0][0] == opm.OPM_OK and got[1][0] == got[0][0] and torch.equal(got[1][1], got[0][1])
