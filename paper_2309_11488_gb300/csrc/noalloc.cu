@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
     if (staged) {
       const int first = __shfl_sync(all, m0, 0);
       const int end = __reduce_max_sync(all, in ? m1 : first);
-      for (int c0 = first; c0 < end; c0 += kNaChunk) {
-        const int cnt = min(kNaChunk, end - c0);
+      for (int64_t c = first; c < end; c += kNaChunk) {  // past the last block, c may not fit an int32
+        const int c0 = (int)c, cnt = min(kNaChunk, end - c0);
         constexpr int kV = (9 * kNaChunk + 31) / 32, kX = (3 * kNaChunk + 31) / 32, kS = (kNaChunk + 31) / 32;
         int col[kX];
 #pragma unroll
