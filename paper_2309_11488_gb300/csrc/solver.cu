@@ -1152,7 +1152,7 @@ opm_status factor_impl(opm_solver *h, const double *vals) {
   if ((s = runner_wait(R)) != OPM_OK) return s;
   CK(cudaEventSynchronize(h->ev[1]));
   cudaEventElapsedTime(&h->timing.factor_ms, h->ev[0], h->ev[1]);
-  h->timing.launches += R.factor_launches;
+  h->timing.launches += R.resident ? 1 : R.factor_launches;
   if (h->opt.profile_kernels) add_kernel_time(h->timing, OPM_KERNEL_FACTOR, h->ev[0], h->ev[1]);
   const Result &r = R.h_res[0];
   if (r.status < 0) {
