@@ -339,14 +339,16 @@ __device__ __forceinline__ bool red_end(double (&v)[NV], RedShared<NV> &rs, cons
   return red_tail<NV>(rs, S, tile, ntiles, nw, lane, tot);
 }
 
-// The second form: a CTA-wide tree in shared memory (values leave the
-// registers at once), then the system's last CTA sums the tile partials in
-// tile order.  k_spmv_t's three sums use it for systems past the resident
-// kernel's sizes (S.tree): at the 949,871-cell system its launch takes 3 us
-// less than with red_end with the product reuse, 10 us less without (an
-// addition per warp costs the FP64 pipe as much as an FMA, and the tree has
-// fewer), while the one- and two-value kernels are faster with red_end
-// (k_spmv_v 135 against 140 us).
+// The second form: CTA-wide, then the system's last CTA sums the tile
+// partials: one counter and one fence between a tile's partial and the sum,
+// where red_end has two of each.  k_spmv_t's three sums use it, in the order
+// of the system (S.tree): a tree in shared memory (values leave the registers
+// at once) and the partials in tile order past the resident kernel's sizes,
+// where its launch takes 3 us less than with red_end at the 949,871-cell
+// system with the product reuse, 10 us less without (an addition per warp
+// costs the FP64 pipe as much as an FMA, and the tree has fewer); red_end's
+// order (last_cta_groups) for the others.  The one- and two-value kernels are
+// faster with red_end (k_spmv_v 135 against 140 us).
 constexpr int kRedThreads = 256;
 
 template <int NV>
@@ -400,6 +402,59 @@ __device__ __forceinline__ bool last_cta_reduce(double (&v)[NV], const Sys &S, i
     for (int q = 0; q < NV; ++q) tot[q] = acc[q];
     S.st->red_count = 0;
   }
+  return true;
+}
+
+// Groups of 32 tiles of the largest system whose sums take red_end's order
+// without the tree (the resident kernel's sizes, two slices per warp of an SM
+// for up to 256 SMs).
+constexpr int kMaxGroups = 64;
+
+// red_end's order with one counter: the tiles' partials from the warps' sums,
+// then the last CTA forms the groups' sums, a group per warp, and the total.
+template <int NV>
+__device__ __forceinline__ bool last_cta_groups(const double (&v)[NV], const Sys &S, int tile, int ntiles,
+                                                double (&tot)[NV]) {
+  __shared__ double wsum[NV][8];
+  __shared__ double gsum[NV][kMaxGroups];
+  __shared__ int amlast;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const double sum = warp_sum_split<NV>(v);
+  const int own = warp_sum_of<NV>(lane);
+  if (own >= 0) wsum[own][wp] = sum;
+  __syncthreads();
+  if (wp == 0) {
+    if (lane < NV) {
+      const double *w = wsum[lane];
+      S.partials[(size_t)tile * NV + lane] = ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) amlast = atomicAdd(&S.st->red_count, 1u) == (unsigned)ntiles - 1;
+  }
+  __syncthreads();
+  if (!amlast) return false;
+  __threadfence();
+  const int ng = (ntiles + 31) >> 5;
+#pragma unroll 1
+  for (int g = wp; g < ng; g += 8) {
+    const int t = 32 * g + lane;
+    double p[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) p[q] = t < ntiles ? __ldcg(S.partials + (size_t)t * NV + q) : 0.0;
+    const double s = warp_sum_split<NV>(p);
+    if (own >= 0) gsum[own][g] = s;
+  }
+  __syncthreads();
+  if (wp != 0) return false;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    tot[q] = 0.0;
+#pragma unroll 1
+    for (int g = lane; g < ng; g += 32) tot[q] += gsum[q][g];
+  }
+  warp_sum<NV>(tot);
+  if (lane == 0) S.st->red_count = 0;
   return true;
 }
 
@@ -738,8 +793,6 @@ enum TreeMode { kTreeNone = 0, kTreeAll = 1, kTreeMixed = 2 };
 // which a small system's latency-bound product prefers.
 template <bool REUSE, bool WIDE, int TREE>
 __global__ void __launch_bounds__(256, (REUSE && !WIDE) ? 6 : 8) k_spmv_t(Batch B) {
-  __shared__ RedShared<3> rs_;
-  if (TREE != kTreeAll) red_begin<3>(rs_);
   pdl_enter();
   OPM_TILE_S(B, S, lt);
   if (!running(S.st)) return;
@@ -760,8 +813,9 @@ __global__ void __launch_bounds__(256, (REUSE && !WIDE) ? 6 : 8) k_spmv_t(Batch 
   }
   double tot[3];
   const bool tree = TREE == kTreeAll || (TREE == kTreeMixed && S.tree);
-  if (tree ? last_cta_reduce<3>(acc, S, lt, S.ntiles_s, tot) && threadIdx.x == 0
-           : red_end<3>(acc, rs_, S, lt, S.ntiles_s, tot) && (threadIdx.x & 31) == 0) {
+  const bool last = tree ? last_cta_reduce<3>(acc, S, lt, S.ntiles_s, tot)
+                         : last_cta_groups<3>(acc, S, lt, S.ntiles_s, tot);
+  if (last && threadIdx.x == 0) {
     DevState *st = S.st;
     st->ts = tot[0];
     st->tt = tot[1];

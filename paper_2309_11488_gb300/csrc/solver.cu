@@ -643,7 +643,9 @@ void runner_destroy(Runner *R) {
 // rows 912, 776, 786; 105,006 rows 1268, 1104, 907; 249,053 rows 1676, 2042,
 // 1309; 354,590 rows 1824, 2707, 1862; 949,871 rows 3482, 6449, 3729.
 bool resident_trios(int nslices, int sms) { return 2 * (int64_t)nslices <= 5 * (int64_t)kTrios * sms; }
-bool resident_size(int nslices, int sms) { return nslices <= 2 * (kResidentThreads / 32) * (int64_t)sms; }
+bool resident_size(int nslices, int sms) {
+  return nslices <= 2 * (kResidentThreads / 32) * (int64_t)sms && nslices <= 256 * kMaxGroups;
+}
 
 // A handle or batch on a stream of its own (not the default stream) is taken
 // to share the device with others.  A resident launch over all SMs would make
