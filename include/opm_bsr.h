@@ -103,7 +103,8 @@ enum {
                                 solves it, with bounded grid barriers between
                                 its stages (on a stream other than the default
                                 one, up to about 18,000 rows and on a quarter
-                                of the SMs, so that streams overlap);
+                                of the SMs, so that streams overlap), where
+                                the number of phases makes it the faster form;
                                 otherwise per-phase launches up to 1024
                                 phases, cooperative sweeps past that.  Every
                                 form gives the same bits                    */

@@ -110,6 +110,7 @@ struct Runner {
   int iter_launches = 0, factor_launches = 0;
   int tree = kTreeNone;   // which systems' sums take the tree's order (Sys::tree)
   bool resident = false;  // factorisation and solve run in the resident kernel
+  bool resident_alone = false;  // and an application alone does
   Resident RA{};          // its arguments
   const void *res_kernel = nullptr, *res_apply = nullptr;
   int res_grid = 1, res_threads = 256;
@@ -647,19 +648,57 @@ bool resident_size(int nslices, int sms) {
   return nslices <= 2 * (kResidentThreads / 32) * (int64_t)sms && nslices <= 256 * kMaxGroups;
 }
 
+// How many phases the resident kernel takes.  Each costs it a grid barrier
+// with a stage's dependent loads behind it, 2.2 to 2.6 us, where a launch of a
+// few slices costs 1.9 and one of hundreds 2.8.  The trio form loads ahead of
+// the barrier; a warp per slice does not, and needs few phases or large ones.
+// Past kMaxPhaseLaunches the launches per phase give way to cooperative ones,
+// at 4 us a phase.  us for refactor + solve to 1e-2 / solve to 1e-8, launches
+// -> resident, FP64 unless said:
+//   trios:   36,000 rows, 128 phases  4611 -> 3820 / 18508 -> 17140
+//            44,431 rows, 116 phases  3554 -> 2430 / 30845 -> 28147
+//            20,000 rows, 299 phases  8688 -> 8018 / 36773 -> 38741
+//            5,600 rows, 704 phases, FP32  15460 -> 13912 / 62635 -> 63786
+//   warps:   62,000 rows, 5 phases     909 ->  863 /  2898 ->  2387
+//            62,000 rows, 7 phases    1107 -> 1221 /  3302 ->  3255; FP32 909 -> 858 / 2527 -> 2480
+//            150,000 rows, 8 phases   1771 -> 1958 /  5363 ->  4849; FP32 1654 -> 1417 / 4707 -> 3933
+//            300,000 rows, 7 phases   2025 -> 1776 /  6894 ->  5569
+//            86,518 rows, 22 phases   1285 -> 1899 / 17885 -> 25904; FP32 1182 -> 1462 / 13786 -> 26318
+//            205,187 rows, 250 phases 11782 -> 20837 / 63488 -> 130883
+//   1,218 phases, 120,000 rows (warps) 97497 -> 78925; 2,004 phases, 16,000 rows 126072 -> 55155
+bool resident_phases(int nphases, int nslices, bool trio, bool fp32) {
+  if (nphases > kMaxPhaseLaunches) return true;
+  return trio ? nphases <= 192 : nphases <= (fp32 ? 8 : 5) || nslices >= 1000 * (int64_t)nphases;
+}
+
+// The same for an application alone, which has the phases' stages and nothing
+// else, launches -> resident: trios, FP64, 128 phases 655 -> 638, 299 phases
+// 1255 -> 1408; FP32, 17 phases 98.5 -> 92.4, 23 phases 112.1 -> 113.8, 116
+// phases 470 -> 552; warps, 3 phases of 733 slices 59.4 -> 58.1, 5 of 388
+// 103 -> 133, 5 of 1,875 195 -> 170, 7 of 1,339 236 -> 240 (FP32 158 -> 171).
+bool resident_apply(int nphases, int nslices, bool trio, bool fp32) {
+  if (nphases > kMaxPhaseLaunches) return true;
+  return trio ? nphases <= (fp32 ? 20 : 192) : nphases <= 3 || nslices >= 1500 * (int64_t)nphases;
+}
+
 // A handle or batch on a stream of its own (not the default stream) is taken
 // to share the device with others.  A resident launch over all SMs would make
 // theirs wait for its whole solve, so it takes a quarter of the SMs, up to
-// three slices per trio (18,240 rows on 152 SMs); larger systems keep the
-// launches per phase, which overlap.  us per solve (FP64, rtol 1e-2) with 1, 2,
-// 4 and 8 handles on as many streams, launches per phase / all SMs / a quarter:
+// three slices per trio (18,240 rows on 152 SMs), or two (12,160 rows) for two
+// phases, which take few launches; larger systems keep the launches per phase,
+// which overlap.  us per solve (FP64, rtol 1e-2) with 1, 2, 4 and 8 handles on
+// as many streams, launches per phase / all SMs / a quarter:
 //    3,868 rows  627 334 202 180 / 390 382 380 379 /  401 207 108 103
 //    7,574 rows  872 485 279 258 / 457 453 450 449 /  582 297 152 150
 //   18,671 rows  961 600 370 322 / 531 520 522 534 /  947 487 258 257
 //   44,431 rows  898 689 439 379 / 605 615 615 612 / 1604 844 438 435
 //  249,053 rows 2208 1522 1121 1121 / 1698 1691 1683 1684 / 4542 2321 1203 1200
+// and one handle of two phases, launches / a quarter: 12,000 rows 205 / 192,
+// 15,000 rows 212 / 248, 17,576 rows 284 / 298.
 int quarter(int sms) { return (sms + 3) / 4; }
-bool shares_device(int nslices, int sms) { return nslices <= 3 * kTrios * quarter(sms); }
+bool shares_device(int nslices, int nphases, int sms) {
+  return nslices <= (nphases > 2 ? 3 : 2) * kTrios * quarter(sms);
+}
 
 // A system's order of summation follows from its size and the sweeps alone,
 // so it is the same in every launch form, alone and in a batch.
@@ -700,9 +739,11 @@ const void *resident_kernel(bool trio, bool apply) {
 // Whether the runner's system goes to the resident kernel, and its work lists.
 opm_status resident_create(Runner &R, int max_entries) {
   if (R.nsys > 1 || R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(R.nall, R.sms)) return OPM_OK;
-  if (R.stream && !shares_device(R.nall, R.sms)) return OPM_OK;
+  if (R.stream && !shares_device(R.nall, R.nphases, R.sms)) return OPM_OK;
   if (R.mem[0]->an.max_chain > kResidentChain) return OPM_OK;
   const bool trio = resident_trios(R.nall, R.sms);
+  if (!resident_phases(R.nphases, R.nall, trio, R.fp32)) return OPM_OK;
+  R.resident_alone = resident_apply(R.nphases, R.nall, trio, R.fp32);
   R.res_kernel = R.fp32 ? resident_kernel<float>(trio, false) : resident_kernel<double>(trio, false);
   R.res_apply = R.fp32 ? resident_kernel<float>(trio, true) : resident_kernel<double>(trio, true);
   R.res_threads = trio ? kTrioThreads : kResidentThreads;
@@ -2031,7 +2072,7 @@ opm_status opm_ilu_apply(opm_handle h, const double *r, double *z) {
   Runner &R = *h->run;
   // the resident kernel reads r and writes z in the caller's order (no gather
   // and scatter passes): z may take r's place, but not overlap it otherwise
-  if (R.resident && (h->sys.b_in == h->sys.x_out || !overlap(h->sys.b_in, h->sys.x_out, h->n))) {
+  if (R.resident && R.resident_alone && (h->sys.b_in == h->sys.x_out || !overlap(h->sys.b_in, h->sys.x_out, h->n))) {
     if ((s = resident_enqueue(R, kResApply)) != OPM_OK) return s;
     h->timing.launches += 1;
   } else {

@@ -24,3 +24,77 @@ def test_launches_are_counted():
             call()
             seen.append(sv.timing().launches)
         assert seen == [1, 2, 3, 4, 5]
+
+
+# (system, schedule, partitions, precision): whether the resident kernel solves it, and applies it alone; by phases
+ROUTES = [
+    (lambda: synth.config3(14), "level", 0, "fp64", True, True),  # 47 phases, trios
+    (lambda: synth.config3(14), "level", 0, "fp32", True, False),
+    (lambda: synth.config3(14), "auto", 0, "fp32", True, True),
+    (lambda: synth.chain_system(300), "natural", 0, "fp64", False, False),  # 300 phases
+    (lambda: synth.chain_system(1025), "natural", 0, "fp32", True, True),  # more than launches are made for
+    (lambda: synth.config3(45), "auto", 0, "fp64", True, True),  # 3 phases, a warp per slice
+    (lambda: synth.config3(45), "level", 512, "fp64", False, False),  # 22 phases
+]
+
+
+@pytest.mark.parametrize("make, schedule, parts, precision, solves, applies", ROUTES)
+def test_routes_by_phases(make, schedule, parts, precision, solves, applies):
+    """A route is seen in the kernels that a call launches; the bits are those of the launches per phase."""
+    s = make()
+    part = np.ascontiguousarray(synth.partition_grid(s, parts), dtype=np.int32) if parts else None
+    b, v = dev(s.x_true), dev(s.vals)
+    out = []
+    for sweep in ("per_phase", "auto"):
+        with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, schedule=schedule, precision=precision, part=part,
+                        sweep_launch=sweep) as sv:
+            x = torch.empty_like(b)
+            n0 = sv.timing().launches
+            sv.launch(v, b, x, rtol=1e-4)
+            got = sv.wait()
+            n1 = sv.timing().launches
+            z = sv.ilu_apply(b)
+            n2 = sv.timing().launches
+            out.append((got, x, z))
+    assert (n1 - n0 == 1) == solves and (n2 - n1 == 1) == applies
+    assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][2], out[1][2])
+
+
+def test_edges_of_the_three_warp_form():
+    """On both sides of the last size of the three-warp form, on all SMs, with up to 2.5 slices per trio; and the
+    44,431-row mesh.  The limit follows from the number of SMs."""
+    slices = 5 * 5 * torch.cuda.get_device_properties(0).multi_processor_count // 2
+    side = round((32 * slices) ** 0.5 / 8) * 8
+    logk = lambda *d: np.random.default_rng(1).normal(size=d)
+    systems = [synth.config2()]
+    for rows in (32 * slices, 32 * slices + 1):  # chains: any row count
+        systems.append(synth.chain_system(rows))
+    systems.append(synth.grid_system(side, 32 * slices // side, 1, logk(1, 32 * slices // side, side), seed=3))
+    for s in systems:
+        for precision in ("fp64", "fp32"):
+            b, v = dev(s.x_true), dev(s.vals)
+            out = []
+            for sweep in ("per_phase", "auto"):
+                with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, precision=precision, sweep_launch=sweep) as sv:
+                    x = torch.empty_like(b)
+                    sv.launch(v, b, x, rtol=1e-6)
+                    out.append((sv.wait(), x, sv.ilu_apply(b), *map(torch.from_numpy, sv.factors())))
+            assert out[0][0] == out[1][0]
+            assert all(torch.equal(p, q) for p, q in zip(out[0][1:], out[1][1:]))
+
+
+def test_sizes_on_a_stream_of_its_own():
+    """A quarter of the SMs: two slices per trio for two phases, three for more."""
+    trios = 5 * ((torch.cuda.get_device_properties(0).multi_processor_count + 3) // 4)
+    side = torch.cuda.Stream()
+    for make, resident in ((lambda: synth.chain_system(64 * trios), True), (lambda: synth.chain_system(64 * trios + 1), False),
+                           (lambda: synth.config3(26), 521 <= 3 * trios)):  # 16,667 rows, 3 phases
+        s = make()
+        b, v = dev(s.x_true), dev(s.vals)
+        x = torch.empty_like(b)
+        torch.cuda.synchronize()
+        with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, stream=side) as sv:
+            n0 = sv.timing().launches
+            sv.launch(v, b, x)
+            assert sv.wait()[0] == opm.OPM_OK
+            assert (sv.timing().launches - n0 == 1) == resident
