@@ -34,8 +34,10 @@ namespace opm {
 
 enum SweepMode { kModePlain = 0, kModeP = 1, kModeS = 2 };
 
-// One system's device data.  The last group of fields is set per call.
-struct alignas(16) Sys {
+// One system's device data.  The last group of fields is set per call.  Not
+// aligned to 16 bytes: the kernels then load neighbouring fields together and
+// wait for both, 0.06 us per launch of a phase of one slice.
+struct Sys {
   int32_t n, nslices, ntiles, nphases;
   int32_t ntiles_s;  // 256-row tiles of the SpMV kernels
   int32_t tree;      // order of the sums within a tile (see red_end)

@@ -1078,10 +1078,10 @@ __device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &s
   const int phase0 = __ldg(B.fwd_ptr + 1);
   if (threadIdx.x == 0) sm.phase0 = phase0;
   if (c.lane == 0 && c.g < phase0) sm.first[wp] = __ldg(B.ent + c.g);
-  const int4 *src = reinterpret_cast<const int4 *>(B.nsys == 1 ? &R.one : B.sys);
-  int4 *dst = reinterpret_cast<int4 *>(sm.sys);
-  static_assert(sizeof(Sys) % sizeof(int4) == 0, "descriptors are copied in 16-byte pieces");
-  for (int q = threadIdx.x; q < B.nsys * (int)(sizeof(Sys) / sizeof(int4)); q += nt) dst[q] = src[q];
+  const int2 *src = reinterpret_cast<const int2 *>(B.nsys == 1 ? &R.one : B.sys);
+  int2 *dst = reinterpret_cast<int2 *>(sm.sys);
+  static_assert(sizeof(Sys) % sizeof(int2) == 0, "descriptors are copied in 8-byte pieces");
+  for (int q = threadIdx.x; q < B.nsys * (int)(sizeof(Sys) / sizeof(int2)); q += nt) dst[q] = src[q];
   __syncthreads();
   if (threadIdx.x < B.nsys) {
     Scal z{};
