@@ -151,8 +151,10 @@ __device__ __forceinline__ void one_pass_rows(const Sys &S, int sl, bool fz, con
 
 // Eliminates the lane's row with its pivots k < i (Algorithm 2's updates of
 // row i), its blocks being in their factor slots.  All lanes of the warp call
-// it; lanes with !gen only take part in the walk.
-template <typename TF>
+// it; lanes with !gen only take part in the walk.  WAIT: the wait for earlier
+// phases comes here, after the row's bounds, which are constant (0.2 us per
+// launch of a small phase).
+template <typename TF, bool WAIT>
 __device__ __forceinline__ void eliminate_row(const Sys &S, int sl, bool gen, TF *lu) {
   const int lane = threadIdx.x & 31;
   const int s0 = sl * 32;
@@ -163,6 +165,7 @@ __device__ __forceinline__ void eliminate_row(const Sys &S, int sl, bool gen, TF
   const int len = (i < n) ? __ldg(S.l_rp + i + 1) - lrow : 0;
   int base = (s0 < n) ? __ldg(S.l_rp + s0) : 0;
   const int maxlen = __reduce_max_sync(0xffffffffu, gen ? len : 0);
+  if (WAIT) pdl_wait();
   for (int k = 0; k < maxlen; ++k) {
     const unsigned m = __ballot_sync(0xffffffffu, len > k);
     if (gen && len > k) {
@@ -210,17 +213,17 @@ __device__ __forceinline__ void eliminate_row(const Sys &S, int sl, bool gen, TF
 }
 
 // Inverts the row's diagonal block, held in D (in_regs) or in its slot, into
-// the slot; false for a singular block.
-template <typename TF>
-__device__ __forceinline__ bool invert_diagonal(const Sys &S, int sl, bool in_regs, const TF (&D)[9], TF *lu) {
+// the slot; a singular block is noted first.
+template <typename TF, typename Note>
+__device__ __forceinline__ void invert_diagonal(const Sys &S, int sl, bool in_regs, const TF (&D)[9], TF *lu,
+                                                const Note &note) {
   TF *Dp = lu + S.d_off + (int64_t)kSliceVals * sl + (threadIdx.x & 31);
   TF a[9], o[9];
 #pragma unroll
   for (int c = 0; c < 9; ++c) a[c] = in_regs ? D[c] : Dp[32 * c];
-  const bool ok = inv3<TF>(a, o);
+  if (!inv3<TF>(a, o)) note(sl * 32 + (int)(threadIdx.x & 31));
 #pragma unroll
   for (int c = 0; c < 9; ++c) Dp[32 * c] = o[c];
-  return ok;
 }
 
 // ILU0 decomposition (Algorithm 2) of the permuted matrix, phase by phase,
@@ -237,9 +240,9 @@ __device__ __forceinline__ bool invert_diagonal(const Sys &S, int sl, bool in_re
 // copy reads only the caller's values and writes only the phase's own rows,
 // so it overlaps the tail of the previous phase; the elimination, which
 // reads earlier phases' pivots, comes after the wait.
-// Returns false for a lane whose row has a singular pivot.
-template <typename TF, bool ONE_PASS, bool EARLY_COPY = false, bool DREG = true>
-__device__ __forceinline__ bool factor_rows(const Sys &S, int sl, int r0, int r1) {
+// note is called with a row whose pivot is singular.
+template <typename TF, bool ONE_PASS, bool EARLY_COPY = false, bool DREG = true, typename Note>
+__device__ __forceinline__ void factor_rows(const Sys &S, int sl, int r0, int r1, const Note &note) {
   const int lane = threadIdx.x & 31;
   const int i = sl * 32 + lane;
   const bool act = i >= r0 && i < r1;
@@ -251,17 +254,19 @@ __device__ __forceinline__ bool factor_rows(const Sys &S, int sl, int r0, int r1
   if (ONE_PASS && __any_sync(0xffffffffu, fz)) one_pass_rows<TF, DREG>(S, sl, fz, vals_user, lu, D);
   if (__any_sync(0xffffffffu, gen)) {
     copy_row_to_factors<TF>(S, sl, gen, vals_user, lu);
-    if (EARLY_COPY) pdl_wait();
-    eliminate_row<TF>(S, sl, gen, lu);
+    eliminate_row<TF, EARLY_COPY>(S, sl, gen, lu);
   }
-  return !act || invert_diagonal<TF>(S, sl, fz && DREG, D, lu);
+  if (act) invert_diagonal<TF>(S, sl, fz && DREG, D, lu, note);
 }
 
-// Records a singular pivot of the lane's row for the host.
-__device__ __forceinline__ void record_singular(DevState *st, int i) {
-  atomicCAS(&st->error, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
-  atomicMin(&st->err_row, i);
-}
+// Records a singular pivot for the host.
+struct RecordSingular {
+  DevState *st;
+  __device__ __forceinline__ void operator()(int i) const {
+    atomicCAS(&st->error, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
+    atomicMin(&st->err_row, i);
+  }
+};
 
 // One launch per phase, one 32-row slice per warp.  ONE_PASS takes the
 // one-pass walk for the rows that allow it, DREG keeps its diagonal in
@@ -287,8 +292,7 @@ __global__ void __launch_bounds__(256, MINB) k_factor_phase(Batch B, int c) {
   const int4 E = B.ent[e];
   const Sys &S = B.sys[E.x];
   if (S.skip) return;  // warp-uniform: the entry belongs to one system
-  if (!factor_rows<TF, ONE_PASS, !ONE_PASS, DREG>(S, E.y, E.z, E.w))
-    record_singular(S.st, E.y * 32 + (threadIdx.x & 31));
+  factor_rows<TF, ONE_PASS, !ONE_PASS, DREG>(S, E.y, E.z, E.w, RecordSingular{S.st});
 }
 
 template <typename TF>
@@ -302,8 +306,7 @@ __global__ void __launch_bounds__(1024) k_factor(Batch B) {
     for (int e = __ldg(B.fwd_ptr + c) + g; e < e1; e += W) {
       const int4 E = B.ent[e];
       const Sys &S = B.sys[E.x];
-      if (!S.skip && !factor_rows<TF, false>(S, E.y, E.z, E.w))
-        record_singular(S.st, E.y * 32 + (threadIdx.x & 31));
+      if (!S.skip) factor_rows<TF, false>(S, E.y, E.z, E.w, RecordSingular{S.st});
     }
   }
 }

@@ -916,8 +916,8 @@ __device__ __forceinline__ void copy_trio(const ResCtx &c, const Sys &S, int sl)
 
 // eliminate_row and invert_diagonal by a trio: row r of the slice's blocks,
 // whose updates need no other row of them until the inversion.
-template <typename TF>
-__device__ __forceinline__ bool eliminate_trio(ResCtx &c, const Sys &S, int4 E) {
+template <typename TF, typename Note>
+__device__ __forceinline__ void eliminate_trio(ResCtx &c, const Sys &S, int4 E, const Note &note) {
   const int lane = c.lane, r = c.r, sl = E.y, s0 = sl * 32, i = s0 + lane;
   const bool act = i >= E.z && i < E.w;
   TF *lu = static_cast<TF *>(S.lu);
@@ -972,16 +972,15 @@ __device__ __forceinline__ bool eliminate_trio(ResCtx &c, const Sys &S, int4 E) 
   TF a[9], o[9];
 #pragma unroll
   for (int e = 0; e < 9; ++e) a[e] = (TF)ex[e / 3][e % 3][lane];
-  if (!act) return true;
-  const bool ok = inv3<TF>(a, o);
+  if (!act) return;
+  if (!inv3<TF>(a, o) && r == 0) note(i);
 #pragma unroll
   for (int e = 0; e < 3; ++e) Dp[32 * (3 * r + e)] = r == 0 ? o[e] : r == 1 ? o[3 + e] : o[6 + e];
-  return ok || r > 0;
 }
 
 // ------------------------------------------------ the kernel
 
-// A singular pivot of the lane's row.
+// A singular pivot of row i.
 __device__ __forceinline__ void note_singular(int32_t *err, int i) {
   atomicCAS(err, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
   atomicMax(err + 1, 0x7fffffff - i);
@@ -1010,10 +1009,9 @@ __device__ __forceinline__ void resident_factor(ResCtx &c) {
       const int4 E = __ldg(B.ent + e);
       const Sys &S = c.sm.sys[E.x];
       if (S.skip) continue;
-      bool ok;
-      if constexpr (TRIO) ok = eliminate_trio<TF>(c, S, E);
-      else ok = factor_rows<TF, true, false, sizeof(TF) == 4>(S, E.y, E.z, E.w);
-      if (!ok) note_singular(c.R.err + 2 * E.x, E.y * 32 + c.lane);
+      const auto note = [&](int i) { note_singular(c.R.err + 2 * E.x, i); };
+      if constexpr (TRIO) eliminate_trio<TF>(c, S, E, note);
+      else factor_rows<TF, true, false, sizeof(TF) == 4>(S, E.y, E.z, E.w, note);
     }
     c.arrive();
   }
