@@ -104,10 +104,14 @@ enum {
                                 its stages (on a stream other than the default
                                 one, up to about 18,000 rows and on a quarter
                                 of the SMs, so that streams overlap), where
-                                the number of phases makes it the faster form;
-                                otherwise per-phase launches up to 1024
-                                phases, cooperative sweeps past that.  Every
-                                form gives the same bits                    */
+                                the number of phases makes it the faster form.
+                                On the default stream it holds every SM for
+                                the whole solve, and work on other streams
+                                waits for it: give handles that are to overlap
+                                streams of their own, or ask for
+                                OPM_SWEEP_PER_PHASE.  Otherwise per-phase
+                                launches up to 1024 phases, cooperative sweeps
+                                past that.  Every form gives the same bits  */
   OPM_SWEEP_PER_PHASE = 1,   /* one kernel launch per phase                 */
   OPM_SWEEP_COOPERATIVE = 2  /* one cooperative launch walking all phases,
                                 with a bounded grid barrier between them    */
@@ -116,7 +120,8 @@ enum {
 typedef struct opm_options {
   int32_t schedule;      /* OPM_SCHED_*                                       */
   int32_t precision;     /* OPM_PREC_*                                        */
-  void *stream;          /* cudaStream_t to issue work on; NULL = default     */
+  void *stream;          /* cudaStream_t to issue work on; NULL or
+                            cudaStreamLegacy = the legacy default stream      */
   int32_t chunk;         /* BiCGStab iterations per body of the device-side
                             solve loop (the loop condition is tested after
                             each body); 0 = default (2)                      */

@@ -681,8 +681,8 @@ bool resident_apply(int nphases, int nslices, bool trio, bool fp32) {
   return trio ? nphases <= (fp32 ? 20 : 192) : nphases <= 3 || nslices >= 1500 * (int64_t)nphases;
 }
 
-// A handle or batch on a stream of its own (not the default stream) is taken
-// to share the device with others.  A resident launch over all SMs would make
+// A handle or batch on a stream of its own (not the legacy default stream, by
+// NULL or by name) is taken to share the device with others.  A resident launch over all SMs would make
 // theirs wait for its whole solve, so it takes a quarter of the SMs, up to
 // three slices per trio (18,240 rows on 152 SMs), or two (12,160 rows) for two
 // phases, which take few launches; larger systems keep the launches per phase,
@@ -695,6 +695,7 @@ bool resident_apply(int nphases, int nslices, bool trio, bool fp32) {
 //  249,053 rows 2208 1522 1121 1121 / 1698 1691 1683 1684 / 4542 2321 1203 1200
 // and one handle of two phases, launches / a quarter: 12,000 rows 205 / 192,
 // 15,000 rows 212 / 248, 17,576 rows 284 / 298.
+bool own_stream(cudaStream_t st) { return st && st != cudaStreamLegacy; }
 int quarter(int sms) { return (sms + 3) / 4; }
 bool shares_device(int nslices, int nphases, int sms) {
   return nslices <= (nphases > 2 ? 3 : 2) * kTrios * quarter(sms);
@@ -739,7 +740,7 @@ const void *resident_kernel(bool trio, bool apply) {
 // Whether the runner's system goes to the resident kernel, and its work lists.
 opm_status resident_create(Runner &R, int max_entries) {
   if (R.nsys > 1 || R.cp_sweeps > 0 || R.tri_sweeps > 0 || !resident_size(R.nall, R.sms)) return OPM_OK;
-  if (R.stream && !shares_device(R.nall, R.nphases, R.sms)) return OPM_OK;
+  if (own_stream(R.stream) && !shares_device(R.nall, R.nphases, R.sms)) return OPM_OK;
   if (R.mem[0]->an.max_chain > kResidentChain) return OPM_OK;
   const bool trio = resident_trios(R.nall, R.sms);
   if (!resident_phases(R.nphases, R.nall, trio, R.fp32)) return OPM_OK;
@@ -756,7 +757,7 @@ opm_status resident_create(Runner &R, int max_entries) {
       return OPM_OK;
     }
   }
-  const int sms = R.stream ? quarter(R.sms) : R.sms;  // one CTA per SM
+  const int sms = own_stream(R.stream) ? quarter(R.sms) : R.sms;  // one CTA per SM
   R.res_grid = std::max(1, std::min(sms, std::max(max_entries, R.nall)));
   std::vector<int32_t> off_s(1, 0), off_u(1, 0), goff_s(1, 0), goff_u(1, 0);
   std::vector<int2> grp_s, grp_u;

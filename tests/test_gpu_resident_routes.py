@@ -98,3 +98,15 @@ def test_sizes_on_a_stream_of_its_own():
             sv.launch(v, b, x)
             assert sv.wait()[0] == opm.OPM_OK
             assert (sv.timing().launches - n0 == 1) == resident
+
+
+def test_legacy_stream_by_name():
+    """cudaStreamLegacy is the default stream: 44,431 rows are one launch there, and not on a stream of their own."""
+    s = synth.config2()
+    b, v = dev(s.x_true), dev(s.vals)
+    torch.cuda.synchronize()
+    for stream, resident in ((1, True), (torch.cuda.Stream(), False)):
+        with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, stream=stream) as sv:
+            n0 = sv.timing().launches
+            assert sv.solve(b)[1] == opm.OPM_OK
+            assert (sv.timing().launches - n0 == 1) == resident
