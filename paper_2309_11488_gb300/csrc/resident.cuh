@@ -1,5 +1,5 @@
-// The resident kernel: one cooperative launch refactors and solves a set of
-// systems; its CTAs stay on the SMs from the value permutation to the true
+// The resident kernel: one cooperative launch refactors and solves one
+// system; its CTAs stay on the SMs from the value permutation to the true
 // residual.  The phases of the factorisation and of the sweeps, the products
 // and the updates are stages separated by grid barriers with bounded waits.
 //
@@ -46,25 +46,22 @@ struct ResidentCtl {
 // units, grouped by 256.
 struct DotUnits {
   double *sums;
-  const int32_t *off;   // [nsys + 1] first unit of a system
-  const int2 *grp;      // (system, group)
-  const int32_t *goff;  // [nsys + 1] first group of a system
   int32_t ngrp, nunits;
 };
 
 struct Resident {
   Batch B;
-  Sys one;                // the system's descriptor when nsys == 1 (else B.sys)
+  Sys sys;                // the system's descriptor (B.sys is not read)
   ResidentCtl *ctl;
-  int32_t *err;           // [2 nsys] factorisation errors: status, 0x7fffffff - smallest row (both 0: none)
-  const int4 *prod;       // every slice of every system for the products, the heaviest first
+  int32_t *err;           // factorisation error: status, 0x7fffffff - smallest row (both 0: none)
+  const int32_t *prod;    // every slice for the products, the heaviest first
   DotUnits ds, du;        // slice units (whole 256-row tiles), update units (whole 1024-row tiles)
   double *gpart;          // group sums, three values per group
   Result *res;            // the outcome, in page-locked host memory
   int32_t nupd, work;
 };
 
-// Krylov scalars of one system, kept by every CTA in shared memory.
+// The Krylov scalars, kept by every CTA in shared memory.
 struct Scal {
   double n0, tol, rho, alpha, omega, beta, relres;
   double tot[3], part[3];  // a complete sum and the slow parts of its decision
@@ -75,15 +72,13 @@ struct Scal {
 // that was switched out (a time slice, a debugger) has not waited.
 constexpr uint64_t kPollGapNs = 1000000;
 
-constexpr int kResMaxSys = 16;  // systems of one launch (descriptors and scalars in shared memory)
-
 constexpr int kTrios = 5;       // trios of a CTA of the trio form
 constexpr int kTrioThreads = 32 * (3 * kTrios + 1);  // and one warp more: the boss's
 constexpr int kResidentThreads = 1024;               // the wide form
 
 struct ResShared {
-  Sys sys[kResMaxSys];
-  Scal sc[kResMaxSys];
+  Sys sys;  // k_resident_apply's
+  Scal sc;
   int dead, last;
   int32_t phase0;                           // entries of the first forward phase
   int4 first[kResidentThreads / 32];        // the warps' first entry of it
@@ -171,6 +166,7 @@ __device__ __forceinline__ void red_release(uint32_t *p) {
 struct ResCtx {
   const Resident &R;
   ResShared &sm;
+  const Sys &S;      // the system's descriptor
   int lane, wp, nw;  // lane, warp of the CTA, warps per CTA
   int g, W;          // first unit of a stage of this warp (trio), the units' stride
   int r, trio;       // component and trio of the warp (trios only)
@@ -221,8 +217,8 @@ struct ResCtx {
     __syncthreads();
     dead = sm.dead != 0;
   }
-  // Whether system s takes part in an iteration's stages.
-  __device__ __forceinline__ bool runs(int s) const { return !sm.sys[s].skip && sm.sc[s].status == kRunning; }
+  // Whether the iteration goes on.
+  __device__ __forceinline__ bool runs() const { return sm.sc.status == kRunning; }
 };
 
 using First = std::true_type;
@@ -249,26 +245,24 @@ __device__ __forceinline__ void store_unit(const DotUnits &D, int u, const doubl
 }
 
 // Completes a step's dot product after the wait: group sums (red_end's order:
-// the butterflies over a tile's eight units and over 32 tiles), then every
-// system's sum and what it decides, by every CTA for itself, a value and a
-// slow operation per warp.  A single group (one system of up to 8,192 rows)
-// is summed by every CTA; more are spread over the grid, with one more
-// barrier: read by every CTA, the unit sums of a 249,053-row system took
-// 35 us per three-value dot, the barrier 1.3.
+// the butterflies over a tile's eight units and over 32 tiles), then the sum
+// and what it decides, by every CTA for itself, a value and a slow operation
+// per warp.  A single group (a system of up to 8,192 rows) is summed by every
+// CTA; more are spread over the grid, with one more barrier: read by every
+// CTA, the unit sums of a 249,053-row system took 35 us per three-value dot,
+// the barrier 1.3.
 __device__ __forceinline__ void finish_dot(ResCtx &c, int step) {
   const DotUnits &D = (step == kStepSetup || step == kStepUpdate) ? c.R.du : c.R.ds;
-  const int nsys = c.R.B.nsys;
   const bool local = D.ngrp == 1, every = step == kStepSetup || step == kStepFinish;
   const int nv = step == kStepS ? 3 : step == kStepUpdate ? 2 : 1;
   double *gp = c.R.gpart;
+  Scal &sc = c.sm.sc;
 #pragma unroll 1
   for (int q = local ? c.wp : c.warp_id(); q < D.ngrp * nv; q += local ? c.nw : c.warps()) {
     const int grp = q / nv, v = q - grp * nv;
-    const int2 G = nsys == 1 ? make_int2(0, grp) : __ldg(D.grp + grp);
-    const int u0 = (nsys == 1 ? 0 : __ldg(D.off + G.x)) + 256 * G.y + 8 * c.lane;
-    const int u1 = nsys == 1 ? D.nunits : __ldg(D.off + G.x + 1);
+    const int u0 = 256 * grp + 8 * c.lane;
     double t[1] = {0.0};
-    if (u0 < u1) {
+    if (u0 < D.nunits) {
       const double *p = D.sums + (size_t)v * D.nunits + u0;
       double a[8];
 #pragma unroll
@@ -277,7 +271,7 @@ __device__ __forceinline__ void finish_dot(ResCtx &c, int step) {
     }
     warp_sum<1>(t);
     if (c.lane == 0) {
-      if (local) c.sm.sc[0].tot[v] = t[0];
+      if (local) sc.tot[v] = t[0];
       else gp[(size_t)grp * 3 + v] = t[0];
     }
   }
@@ -285,26 +279,19 @@ __device__ __forceinline__ void finish_dot(ResCtx &c, int step) {
     c.arrive();
     c.wait();
 #pragma unroll 1
-    for (int a = c.wp; a < nsys * nv; a += c.nw) {
-      const int s = a / nv, v = a - s * nv;
-      const int g0 = nsys == 1 ? 0 : __ldg(D.goff + s), g1 = nsys == 1 ? D.ngrp : __ldg(D.goff + s + 1);
+    for (int v = c.wp; v < nv; v += c.nw) {
       double t[1] = {0.0};
 #pragma unroll 1
-      for (int q = g0 + c.lane; q < g1; q += 32) t[0] += __ldcg(gp + (size_t)q * 3 + v);
+      for (int q = c.lane; q < D.ngrp; q += 32) t[0] += __ldcg(gp + (size_t)q * 3 + v);
       warp_sum<1>(t);
-      if (c.lane == 0) c.sm.sc[s].tot[v] = t[0];
+      if (c.lane == 0) sc.tot[v] = t[0];
     }
   }
   __syncthreads();
   const int parts = dot_parts(step);
-#pragma unroll 1
-  for (int a = c.wp; a < nsys * parts; a += c.nw) {
-    Scal &sc = c.sm.sc[a / parts];
-    if (c.lane == 0) sc.part[a % parts] = dot_part(step, sc, a % parts);
-  }
+  if (c.wp < parts && c.lane == 0) sc.part[c.wp] = dot_part(step, sc, c.wp);
   __syncthreads();
-  if (threadIdx.x < nsys && !c.sm.sys[threadIdx.x].skip && (every || c.sm.sc[threadIdx.x].status == kRunning))
-    dot_decide(step, c.sm.sc[threadIdx.x]);
+  if (threadIdx.x == 0 && (every || sc.status == kRunning)) dot_decide(step, sc);
   __syncthreads();
 }
 
@@ -335,7 +322,7 @@ __device__ __forceinline__ Vec3<TF> sweep_gather(const void *y, const double *z,
 // application reads and writes the caller's order in place.
 template <typename TF, int MODE>
 __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool second) {
-  const Sys &S = c.sm.sys[E.x];
+  const Sys &S = c.S;
   const int lane = c.lane, sl = E.y, s0 = sl * 32, i = s0 + lane;
   constexpr bool kPlain = MODE == kModePlain;
   TF *y = static_cast<TF *>(S.y);
@@ -358,7 +345,7 @@ __device__ __forceinline__ void sweep_unit(ResCtx &c, int4 E, bool fwd, bool sec
   } else if (act && fwd) {
     Vec3<double> h = load3cg(S.r + 3ll * i);
     const Vec3<double> vo = load3cg(S.v + 3ll * i);
-    const Scal &sc = c.sm.sc[E.x];
+    const Scal &sc = c.sm.sc;
     if (second) {
       const double c1 = sc.alpha;
       h.c0 = fma(-c1, vo.c0, h.c0);
@@ -448,14 +435,14 @@ struct ProductIo {
 // A product's slice: v = A p^ and (r^, v); t = A s^, (t,s), (t,t), (s,s); or
 // the true residual and x back in the caller's order (zeros on failure).
 // row_operator_applied with reuse, row_operator without.
-__device__ __forceinline__ void product_unit(ResCtx &c, int4 E, int step, bool reuse) {
-  const Sys &S = c.sm.sys[E.x];
+__device__ __forceinline__ void product_unit(ResCtx &c, int sl, int step, bool reuse) {
+  const Sys &S = c.S;
   const bool fin = step == kStepFinish;
-  const int status = c.sm.sc[E.x].status;
+  const int status = c.sm.sc.status;
   const bool ok = !fin || status == OPM_OK || status == OPM_NOT_CONVERGED;
   const ProductIo io(S, step);
   reuse = reuse && !fin;
-  const int lane = c.lane, n = S.n, sl = E.y, s0 = sl * 32, i = s0 + lane;
+  const int lane = c.lane, n = S.n, s0 = sl * 32, i = s0 + lane;
   const bool in = i < n;
   const int len = in ? __ldg(S.a_rp + i + 1) - __ldg(S.a_rp + i) : 0;
   const uint2 M = reuse ? __ldg(S.sp_mask + sl) : make_uint2(0u, 0u);
@@ -514,16 +501,14 @@ __device__ __forceinline__ void product_unit(ResCtx &c, int4 E, int step, bool r
       acc[2] = fma(q.c0, q.c0, fma(q.c1, q.c1, fma(q.c2, q.c2, acc[2])));
     }
   }
-  store_unit(c.R.ds, (c.R.B.nsys == 1 ? 0 : __ldg(c.R.ds.off + E.x)) + sl, acc);
+  store_unit(c.R.ds, sl, acc);
 }
 
-// inv(D) B x of every well of every system, one warp per well (k_wells).
+// inv(D) B x of every well, one warp per well (k_wells).
 __device__ __forceinline__ void wells_stage(ResCtx &c, int step) {
   c.wait();
-#pragma unroll 1
-  for (int s = 0; s < c.R.B.nsys && !c.dead; ++s) {
-    const Sys &S = c.sm.sys[s];
-    if (S.skip || (step != kStepFinish && c.sm.sc[s].status != kRunning)) continue;
+  const Sys &S = c.S;
+  if (!c.dead) {
     const double *x = step == kStepFinish ? S.x : step == kStepS ? S.sh : S.ph;
 #pragma unroll 1
     for (int w = c.warp_id(); w < S.nwells; w += c.warps()) {
@@ -551,14 +536,12 @@ __device__ __forceinline__ void wells_stage(ResCtx &c, int step) {
 // Setup unit u (k_setup's rows of one warp: r = r^ = P b, x = p = v = 0 and
 // the unit's part of ||b||^2) or update unit u (k_update's rows).
 __device__ __forceinline__ void vector_unit(ResCtx &c, int u, bool setup) {
-  const int2 T = __ldg(c.R.B.tiles + (u >> 3));
-  const Sys &S = c.sm.sys[T.x];
-  if (S.skip || (!setup && c.sm.sc[T.x].status != kRunning)) return;
-  const double alpha = c.sm.sc[T.x].alpha, omega = c.sm.sc[T.x].omega;
-  const bool half = c.sm.sc[T.x].half;
+  const Sys &S = c.S;
+  const double alpha = c.sm.sc.alpha, omega = c.sm.sc.omega;
+  const bool half = c.sm.sc.half;
   double acc[3] = {0.0, 0.0, 0.0};
 #pragma unroll 1
-  for (int p = 0, i = T.y * kTileRows + (u & 7) * 32 + c.lane; p < 4; ++p, i += 256) {
+  for (int p = 0, i = (u >> 3) * kTileRows + (u & 7) * 32 + c.lane; p < 4; ++p, i += 256) {
     if (i >= S.n) break;
     const size_t e = 3ll * i;
     if (setup) {
@@ -590,7 +573,7 @@ __device__ __forceinline__ void vector_unit(ResCtx &c, int u, bool setup) {
     S.x[e + 1] = fma(alpha, ph.c1, x.c1);
     S.x[e + 2] = fma(alpha, ph.c2, x.c2);
   }
-  if (setup || !half) store_unit(c.R.du, (c.R.B.nsys == 1 ? 0 : __ldg(c.R.du.off + T.x)) + 8 * T.y + (u & 7), acc);
+  if (setup || !half) store_unit(c.R.du, u, acc);
 }
 
 // ------------------------------------------------ units of three warps
@@ -638,7 +621,7 @@ __device__ __forceinline__ int preload_row(const int32_t *col, const T *vals, in
 // sweep_unit by a trio; FIRST: wait() is called here.
 template <typename TF, int MODE, bool FIRST>
 __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool second) {
-  const Sys &S = c.sm.sys[E.x];
+  const Sys &S = c.S;
   const int lane = c.lane, r = c.r, sl = E.y, s0 = sl * 32, i = s0 + lane;
   constexpr bool kPlain = MODE == kModePlain;
   TF *y = static_cast<TF *>(S.y);
@@ -689,7 +672,7 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
   if (act && fwd && kPlain) {
     a = (TF)h;
   } else if (act && fwd) {
-    const Scal &sc = c.sm.sc[E.x];
+    const Scal &sc = c.sm.sc;
     h = second ? fma(-sc.alpha, vo, h) : fma(sc.beta, fma(-sc.omega, vo, po), h);
     (second ? S.s : S.p)[e] = h;
     a = (TF)h;
@@ -730,14 +713,14 @@ __device__ __forceinline__ void sweep_trio(ResCtx &c, int4 E, bool fwd, bool sec
 
 // product_unit by a trio; FIRST: wait() is called here.
 template <bool FIRST>
-__device__ __forceinline__ void product_trio(ResCtx &c, int4 E, int step, bool reuse) {
-  const Sys &S = c.sm.sys[E.x];
+__device__ __forceinline__ void product_trio(ResCtx &c, int sl, int step, bool reuse) {
+  const Sys &S = c.S;
   const bool fin = step == kStepFinish;
-  const int status = c.sm.sc[E.x].status;
+  const int status = c.sm.sc.status;
   const bool ok = !fin || status == OPM_OK || status == OPM_NOT_CONVERGED;
   const ProductIo io(S, step);
   reuse = reuse && !fin;
-  const int lane = c.lane, r = c.r, n = S.n, sl = E.y, s0 = sl * 32, i = s0 + lane;
+  const int lane = c.lane, r = c.r, n = S.n, s0 = sl * 32, i = s0 + lane;
   const bool in = i < n;
   const int len = in ? __ldg(S.a_rp + i + 1) - __ldg(S.a_rp + i) : 0;
   const uint2 M = reuse ? __ldg(S.sp_mask + sl) : make_uint2(0u, 0u);
@@ -798,18 +781,15 @@ __device__ __forceinline__ void product_trio(ResCtx &c, int4 E, int step, bool r
     v[0] = fma(f.c0, g.c0, fma(f.c1, g.c1, fma(f.c2, g.c2, v[0])));
   }
   warp_sum<1>(v);
-  if (lane == 0)
-    c.R.ds.sums[(size_t)r * c.R.ds.nunits + (c.R.B.nsys == 1 ? 0 : __ldg(c.R.ds.off + E.x)) + sl] = v[0];
+  if (lane == 0) c.R.ds.sums[(size_t)r * c.R.ds.nunits + sl] = v[0];
 }
 
 // vector_unit by a trio.
 __device__ __forceinline__ void vector_trio(ResCtx &c, int u, bool setup) {
-  const int2 T = __ldg(c.R.B.tiles + (u >> 3));
-  const Sys &S = c.sm.sys[T.x];
-  if (S.skip || (!setup && c.sm.sc[T.x].status != kRunning)) return;
-  const double alpha = c.sm.sc[T.x].alpha, omega = c.sm.sc[T.x].omega;
-  const bool half = c.sm.sc[T.x].half;
-  const int lane = c.lane, r = c.r, i0 = T.y * kTileRows + (u & 7) * 32 + lane;
+  const Sys &S = c.S;
+  const double alpha = c.sm.sc.alpha, omega = c.sm.sc.omega;
+  const bool half = c.sm.sc.half;
+  const int lane = c.lane, r = c.r, i0 = (u >> 3) * kTileRows + (u & 7) * 32 + lane;
   double(*ex)[3][32] = c.sm.ex[c.trio][c.flip];
   c.flip ^= 1;
   double x[4], ph[4], sh[4], t[4], s[4];
@@ -872,9 +852,7 @@ __device__ __forceinline__ void vector_trio(ResCtx &c, int u, bool setup) {
     }
   }
   warp_sum<1>(acc);
-  if (lane == 0)
-    c.R.du.sums[(size_t)r * c.R.du.nunits + (c.R.B.nsys == 1 ? 0 : __ldg(c.R.du.off + T.x)) + 8 * T.y + (u & 7)] =
-        acc[0];
+  if (lane == 0) c.R.du.sums[(size_t)r * c.R.du.nunits + u] = acc[0];
 }
 
 // copy_row_to_factors by a trio: row r of every block of slice sl.
@@ -980,7 +958,7 @@ __device__ __forceinline__ void eliminate_trio(ResCtx &c, const Sys &S, int4 E, 
 
 // ------------------------------------------------ the kernel
 
-// A singular pivot of row i.
+// A singular pivot of the lane's row.
 __device__ __forceinline__ void note_singular(int32_t *err, int i) {
   atomicCAS(err, 0, (int32_t)OPM_ERR_ZERO_PIVOT);
   atomicMax(err + 1, 0x7fffffff - i);
@@ -994,10 +972,7 @@ __device__ __forceinline__ void resident_factor(ResCtx &c) {
   const Batch &B = c.R.B;
   if (TRIO) {
 #pragma unroll 1
-    for (int u = c.g; u < B.nall; u += c.W) {
-      const int4 E = __ldg(B.all_ent + u);
-      if (!c.sm.sys[E.x].skip) copy_trio<TF>(c, c.sm.sys[E.x], E.y);
-    }
+    for (int sl = c.g; sl < B.nall; sl += c.W) copy_trio<TF>(c, c.S, sl);
     c.arrive();
   }
 #pragma unroll 1
@@ -1007,17 +982,15 @@ __device__ __forceinline__ void resident_factor(ResCtx &c) {
 #pragma unroll 1
     for (int e = __ldg(B.fwd_ptr + p) + c.g; e < e1 && !c.dead; e += c.W) {
       const int4 E = __ldg(B.ent + e);
-      const Sys &S = c.sm.sys[E.x];
-      if (S.skip) continue;
-      const auto note = [&](int i) { note_singular(c.R.err + 2 * E.x, i); };
+      const Sys &S = c.S;
+      const auto note = [&](int i) { note_singular(c.R.err, i); };
       if constexpr (TRIO) eliminate_trio<TF>(c, S, E, note);
       else factor_rows<TF, true, false, sizeof(TF) == 4>(S, E.y, E.z, E.w, note);
     }
     c.arrive();
   }
   c.wait();
-  for (int s = threadIdx.x; s < B.nsys; s += blockDim.x)
-    if (!c.sm.sys[s].skip && __ldcg(c.R.err + 2 * s) != 0) c.sm.sc[s].status = OPM_ERR_ZERO_PIVOT;
+  if (threadIdx.x == 0 && __ldcg(c.R.err) != 0) c.sm.sc.status = OPM_ERR_ZERO_PIVOT;
   __syncthreads();
 }
 
@@ -1032,7 +1005,6 @@ __device__ __forceinline__ void resident_apply(ResCtx &c, bool second) {
 #pragma unroll 1
   for (int e = c.g, e1 = c.sm.phase0; e < e1; e += c.W) {
     const int4 E = e == c.g ? c.sm.first[c.wp] : __ldg(B.ent + e);
-    if (!c.runs(E.x)) continue;
     if constexpr (TRIO) sweep_trio<TF, MODE, false>(c, E, true, second);
     else sweep_unit<TF, MODE>(c, E, true, second);
   }
@@ -1048,22 +1020,24 @@ __device__ __forceinline__ void resident_apply(ResCtx &c, bool second) {
     stage(c, e0, e1, [&](int e, auto first) {
       constexpr bool F = decltype(first)::value;
       const int4 E = __ldg(B.ent + e);
-      const bool run = c.runs(E.x);
-      if (F && (!TRIO || !run)) c.wait();
-      if (!run) return;
+      if (F && !TRIO) c.wait();
       if constexpr (TRIO) sweep_trio<TF, MODE, F>(c, E, fwd, second);
       else sweep_unit<TF, MODE>(c, E, fwd, second);
     });
   }
 }
 
-// The start of a launch: descriptors and scalars into shared memory, and the
-// warp's place among the units.
-template <bool TRIO>
+// The start of a launch: the scalars into shared memory, and the warp's place
+// among the units.  COPY: the descriptor too.  A solve reads it where it is, in
+// the launch's parameters (FP64, 44,431 rows: 307 us against 316 from shared
+// memory; 116 phases 2306 against 2467); an application alone would wait for
+// its fields one after the other (45 us against 42).
+template <bool TRIO, bool COPY>
 __device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &sm) {
   const Batch &B = R.B;
   const int wp = threadIdx.x >> 5, nt = blockDim.x;
-  ResCtx c{R, sm, (int)(threadIdx.x & 31), wp, nt / 32, 0, 0, 0, 0, 0, 0u, false, (int)threadIdx.x == nt - 32};
+  ResCtx c{R, sm, COPY ? sm.sys : R.sys, (int)(threadIdx.x & 31), wp, nt / 32, 0, 0, 0, 0, 0, 0u, false,
+           (int)threadIdx.x == nt - 32};
   if (TRIO) {
     c.r = wp % 3;
     c.trio = wp / 3;
@@ -1076,20 +1050,20 @@ __device__ __forceinline__ ResCtx resident_enter(const Resident &R, ResShared &s
   const int phase0 = __ldg(B.fwd_ptr + 1);
   if (threadIdx.x == 0) sm.phase0 = phase0;
   if (c.lane == 0 && c.g < phase0) sm.first[wp] = __ldg(B.ent + c.g);
-  const int2 *src = reinterpret_cast<const int2 *>(B.nsys == 1 ? &R.one : B.sys);
-  int2 *dst = reinterpret_cast<int2 *>(sm.sys);
-  static_assert(sizeof(Sys) % sizeof(int2) == 0, "descriptors are copied in 8-byte pieces");
-  for (int q = threadIdx.x; q < B.nsys * (int)(sizeof(Sys) / sizeof(int2)); q += nt) dst[q] = src[q];
-  __syncthreads();
-  if (threadIdx.x < B.nsys) {
+  if (COPY) {
+    const int2 *src = reinterpret_cast<const int2 *>(&R.sys);
+    int2 *dst = reinterpret_cast<int2 *>(&sm.sys);
+    static_assert(sizeof(Sys) % sizeof(int2) == 0, "the descriptor is copied in 8-byte pieces");
+    for (int q = threadIdx.x; q < (int)(sizeof(Sys) / sizeof(int2)); q += nt) dst[q] = src[q];
+  }
+  if (threadIdx.x == 0) {
     Scal z{};
-    const Sys &S = sm.sys[threadIdx.x];
-    z.tol = S.rtol;
-    z.maxit = S.maxit;
+    z.tol = R.sys.rtol;
+    z.maxit = R.sys.maxit;
     // an earlier factorisation's failure makes the solve fail
-    const int32_t ferr = (R.work == kResSolve && !S.skip) ? S.st->ferror : 0;
-    z.status = ferr != 0 ? ferr : S.skip ? OPM_OK : kRunning;
-    sm.sc[threadIdx.x] = z;
+    const int32_t ferr = R.work == kResSolve ? R.sys.st->ferror : 0;
+    z.status = ferr != 0 ? ferr : kRunning;
+    sm.sc = z;
   }
   __syncthreads();
   return c;
@@ -1111,35 +1085,28 @@ __device__ __forceinline__ void resident_leave(ResCtx &c) {
   __syncthreads();
   if (!sm.last) return;
   const bool aborted = ld_acquire(&R.ctl->abort) != 0u;
+  const Sys &S = R.sys;
   if (aborted && solve)
-    for (int s = 0; s < R.B.nsys; ++s)
-      for (int64_t e = threadIdx.x; !sm.sys[s].skip && e < 3ll * sm.sys[s].n; e += blockDim.x)
-        sm.sys[s].x_out[e] = 0.0;
-  for (int s = threadIdx.x; s < R.B.nsys; s += blockDim.x) {
-    const Sys &S = sm.sys[s];
-    const Scal &sc = sm.sc[s];
-    if (!S.skip) {
-      const int32_t ferr = __ldcg(R.err + 2 * s);
-      DevState *st = S.st;
-      Result r{};
-      r.status = aborted ? (int32_t)OPM_ERR_TIMEOUT : solve ? sc.status : ferr;  // 0 after an application
-      r.iters = sc.iters;
-      r.relres = aborted ? nan("") : sc.relres;
-      r.err_row = ferr != 0 ? 0x7fffffff - __ldcg(R.err + 2 * s + 1) : 0x7fffffff;
-      if (factor) {
-        st->ferror = aborted ? (int32_t)OPM_ERR_TIMEOUT : ferr;
-        st->err_row = r.err_row;
-      }
-      if (factor || solve) {
-        st->error = aborted ? (int32_t)OPM_ERR_TIMEOUT : 0;
-        st->status = r.status;
-      }
-      R.res[s] = r;
-    }
-    R.err[2 * s] = 0;
-    R.err[2 * s + 1] = 0;
-  }
+    for (int64_t e = threadIdx.x; e < 3ll * S.n; e += blockDim.x) S.x_out[e] = 0.0;
   if (threadIdx.x == 0) {
+    const int32_t ferr = __ldcg(R.err);
+    DevState *st = S.st;
+    Result r{};
+    r.status = aborted ? (int32_t)OPM_ERR_TIMEOUT : solve ? sm.sc.status : ferr;  // 0 after an application
+    r.iters = sm.sc.iters;
+    r.relres = aborted ? nan("") : sm.sc.relres;
+    r.err_row = ferr != 0 ? 0x7fffffff - __ldcg(R.err + 1) : 0x7fffffff;
+    if (factor) {
+      st->ferror = aborted ? (int32_t)OPM_ERR_TIMEOUT : ferr;
+      st->err_row = r.err_row;
+    }
+    if (factor || solve) {
+      st->error = aborted ? (int32_t)OPM_ERR_TIMEOUT : 0;
+      st->status = r.status;
+    }
+    *R.res = r;
+    R.err[0] = 0;
+    R.err[1] = 0;
     R.ctl->arrive = 0;
     R.ctl->exits = 0;
     R.ctl->abort = 0;
@@ -1150,7 +1117,7 @@ __device__ __forceinline__ void resident_leave(ResCtx &c) {
 template <typename TF, bool TRIO, int NT>
 __global__ void __launch_bounds__(NT, 1) k_resident_apply(const __grid_constant__ Resident R) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  ResCtx c = resident_enter<TRIO>(R, *reinterpret_cast<ResShared *>(smem_raw));
+  ResCtx c = resident_enter<TRIO, true>(R, *reinterpret_cast<ResShared *>(smem_raw));
   resident_apply<TF, kModePlain, TRIO>(c, false);
   resident_leave(c);
 }
@@ -1164,13 +1131,9 @@ __global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resi
   ResShared &sm = *reinterpret_cast<ResShared *>(smem_raw);
   const Batch &B = R.B;
   static_assert(!TRIO || NT == kTrioThreads, "the trios and one warp more");
-  ResCtx c = resident_enter<TRIO>(R, sm);
+  ResCtx c = resident_enter<TRIO, false>(R, sm);
   const bool factor = R.work & kResFactor, solve = R.work & kResSolve;
-  bool wells = false, reuse = false;
-  for (int s = 0; s < B.nsys; ++s) {
-    wells = wells || (sm.sys[s].nwells > 0 && !sm.sys[s].skip);
-    reuse = reuse || sm.sys[s].uz != nullptr;
-  }
+  const bool wells = R.sys.nwells > 0, reuse = R.sys.uz != nullptr;
   auto vector_stage = [&](bool setup) {
 #pragma unroll 1
     for (int u = c.g; u < R.nupd; u += c.W) {
@@ -1205,21 +1168,17 @@ __global__ void __launch_bounds__(NT, 1) k_resident(const __grid_constant__ Resi
       if (wells && !c.dead) wells_stage(c, step);
       stage(c, 0, B.nall, [&](int u, auto first) {
         constexpr bool F = decltype(first)::value;
-        const int4 E = __ldg(R.prod + u);
-        const bool run = step == kStepFinish ? !sm.sys[E.x].skip : c.runs(E.x);
-        if (F && (!TRIO || !run)) c.wait();
-        if (!run) return;
-        if constexpr (TRIO) product_trio<F>(c, E, step, reuse);
-        else product_unit(c, E, step, reuse);
+        const int sl = __ldg(R.prod + u);
+        if (F && !TRIO) c.wait();
+        if constexpr (TRIO) product_trio<F>(c, sl, step, reuse);
+        else product_unit(c, sl, step, reuse);
       });
     }
     if (step != kStepSetup) c.wait();
     if (c.dead) break;
     finish_dot(c, step);
     if (step == kStepFinish) break;
-    bool any = false;
-    for (int s = 0; s < B.nsys; ++s) any = any || c.runs(s);
-    step = !any ? kStepFinish : step == kStepP ? kStepS : step == kStepS ? kStepUpdate : kStepP;
+    step = !c.runs() ? kStepFinish : step == kStepP ? kStepS : step == kStepS ? kStepUpdate : kStepP;
   }
 
   resident_leave(c);

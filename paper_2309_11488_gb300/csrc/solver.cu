@@ -682,12 +682,13 @@ bool resident_apply(int nphases, int nslices, bool trio, bool fp32) {
 }
 
 // A handle or batch on a stream of its own (not the legacy default stream, by
-// NULL or by name) is taken to share the device with others.  A resident launch over all SMs would make
-// theirs wait for its whole solve, so it takes a quarter of the SMs, up to
-// three slices per trio (18,240 rows on 152 SMs), or two (12,160 rows) for two
-// phases, which take few launches; larger systems keep the launches per phase,
-// which overlap.  us per solve (FP64, rtol 1e-2) with 1, 2, 4 and 8 handles on
-// as many streams, launches per phase / all SMs / a quarter:
+// NULL or by name) is taken to share the device with others.  A resident
+// launch over all SMs would make theirs wait for its whole solve, so it takes a
+// quarter of the SMs, up to three slices per trio (18,240 rows on 152 SMs), or
+// two (12,160 rows) for two phases, which take few launches; larger systems
+// keep the launches per phase, which overlap.  us per solve (FP64, rtol 1e-2)
+// with 1, 2, 4 and 8 handles on as many streams, launches per phase / all SMs /
+// a quarter:
 //    3,868 rows  627 334 202 180 / 390 382 380 379 /  401 207 108 103
 //    7,574 rows  872 485 279 258 / 457 453 450 449 /  582 297 152 150
 //   18,671 rows  961 600 370 322 / 531 520 522 534 /  947 487 258 257
@@ -759,69 +760,42 @@ opm_status resident_create(Runner &R, int max_entries) {
   }
   const int sms = own_stream(R.stream) ? quarter(R.sms) : R.sms;  // one CTA per SM
   R.res_grid = std::max(1, std::min(sms, std::max(max_entries, R.nall)));
-  std::vector<int32_t> off_s(1, 0), off_u(1, 0), goff_s(1, 0), goff_u(1, 0);
-  std::vector<int2> grp_s, grp_u;
-  for (int s = 0; s < R.nsys; ++s) {
-    const Sys &S = R.mem[s]->sys;
-    off_s.push_back(off_s.back() + 8 * S.ntiles_s);
-    off_u.push_back(off_u.back() + 8 * S.ntiles);
-    for (int g = 0; g < (S.ntiles_s + 31) / 32; ++g) grp_s.push_back(make_int2(s, g));
-    for (int g = 0; g < (S.ntiles + 31) / 32; ++g) grp_u.push_back(make_int2(s, g));
-    goff_s.push_back((int32_t)grp_s.size());
-    goff_u.push_back((int32_t)grp_u.size());
+  // slices of the products, those of the heaviest 256-row tiles first: dealt
+  // round robin over the warps, the last round is then the cheapest
+  const opm_solver &h = *R.mem[0];
+  const Analysis &an = h.an;
+  std::vector<int32_t> prod(h.nslices);
+  std::vector<int64_t> work(h.sys.ntiles_s);
+  for (int t = 0; t < h.sys.ntiles_s; ++t) {
+    const int r0 = t * kSpmvRows, r1 = std::min(an.n, r0 + kSpmvRows);
+    work[t] = R.reuse && t < (int)an.sp_tile.size() ? an.sp_tile[t] : an.a_rowptr[r1] - an.a_rowptr[r0];
   }
-  // units of the products, heaviest 256-row tiles first: dealt round robin
-  // over the warps, the last round is then the cheapest
-  std::vector<int4> prod;
-  std::vector<int64_t> work;
-  for (int s = 0; s < R.nsys; ++s) {
-    const Analysis &an = R.mem[s]->an;
-    for (int sl = 0; sl < R.mem[s]->nslices; ++sl) {
-      const int t = sl / 8, r0 = t * kSpmvRows, r1 = std::min(an.n, r0 + kSpmvRows);
-      prod.push_back(make_int4(s, sl, 0, an.n));
-      work.push_back(R.reuse && t < (int)an.sp_tile.size() ? an.sp_tile[t] : an.a_rowptr[r1] - an.a_rowptr[r0]);
-    }
-  }
-  {
-    std::vector<int> ord(prod.size());
-    for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int)q;
-    std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return work[a] > work[b]; });
-    std::vector<int4> sorted(prod.size());
-    for (size_t q = 0; q < ord.size(); ++q) sorted[q] = prod[ord[q]];
-    prod.swap(sorted);
-  }
+  for (int sl = 0; sl < h.nslices; ++sl) prod[sl] = sl;
+  std::stable_sort(prod.begin(), prod.end(), [&](int a, int b) { return work[a / 8] > work[b / 8]; });
   Resident &A = R.RA;
-  int4 *d_prod;
-  if (opm_status sp = upload(R.allocs, R.dev_bytes, R.stream, &d_prod, prod); sp != OPM_OK) return sp;
-  A.prod = d_prod;
-  int32_t *d_os, *d_ou, *d_gos, *d_gou;
-  int2 *d_gs, *d_gu;
+  int32_t *d_prod;
   opm_status s;
-  if ((s = upload(R.allocs, R.dev_bytes, R.stream, &d_os, off_s)) != OPM_OK ||
-      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_ou, off_u)) != OPM_OK ||
-      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gos, goff_s)) != OPM_OK ||
-      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gou, goff_u)) != OPM_OK ||
-      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gs, grp_s)) != OPM_OK ||
-      (s = upload(R.allocs, R.dev_bytes, R.stream, &d_gu, grp_u)) != OPM_OK)
-    return s;
-  const size_t ns = (size_t)off_s.back(), nu = (size_t)off_u.back();
+  if ((s = upload(R.allocs, R.dev_bytes, R.stream, &d_prod, prod)) != OPM_OK) return s;
+  A.prod = d_prod;
+  const int ns = 8 * h.sys.ntiles_s, nu = 8 * h.sys.ntiles;
+  const int gs = (h.sys.ntiles_s + 31) / 32, gu = (h.sys.ntiles + 31) / 32;
   double *sum_s, *sum_u;
-  if ((s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_s, 3 * ns)) != OPM_OK ||
-      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_u, 3 * nu)) != OPM_OK ||
-      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.gpart, 3 * std::max(grp_s.size(), grp_u.size()))) != OPM_OK ||
-      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.err, 2 * (size_t)R.nsys)) != OPM_OK ||
+  if ((s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_s, 3 * (size_t)ns)) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &sum_u, 3 * (size_t)nu)) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.gpart, 3 * (size_t)std::max(gs, gu))) != OPM_OK ||
+      (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.err, 2)) != OPM_OK ||
       (s = dalloc(R.allocs, R.dev_bytes, R.stream, &A.ctl, 1)) != OPM_OK)
     return s;
-  // the last tile of a system may have fewer than eight slices: the units
-  // past them stay zero
-  CK(cudaMemsetAsync(sum_s, 0, sizeof(double) * 3 * ns, R.stream));
-  CK(cudaMemsetAsync(sum_u, 0, sizeof(double) * 3 * nu, R.stream));
-  CK(cudaMemsetAsync(A.err, 0, sizeof(int32_t) * 2 * R.nsys, R.stream));
+  // the last tile may have fewer than eight slices: the units past them stay
+  // zero
+  CK(cudaMemsetAsync(sum_s, 0, sizeof(double) * 3 * (size_t)ns, R.stream));
+  CK(cudaMemsetAsync(sum_u, 0, sizeof(double) * 3 * (size_t)nu, R.stream));
+  CK(cudaMemsetAsync(A.err, 0, sizeof(int32_t) * 2, R.stream));
   CK(cudaMemsetAsync(A.ctl, 0, sizeof(ResidentCtl), R.stream));
   A.B = R.B;
   A.B.spin_limit_ns = std::max(R.B.spin_limit_ns, kResidentWaitNs);
-  A.ds = {sum_s, d_os, d_gs, d_gos, (int)grp_s.size(), off_s.back()};
-  A.du = {sum_u, d_ou, d_gu, d_gou, (int)grp_u.size(), off_u.back()};
+  A.ds = {sum_s, gs, ns};
+  A.du = {sum_u, gu, nu};
   A.nupd = 8 * R.ntiles;
   A.res = R.h_res;
   R.resident = true;
@@ -830,9 +804,11 @@ opm_status resident_create(Runner &R, int max_entries) {
 
 // Enqueues the resident kernel (work: bits of ResidentWork).
 opm_status resident_enqueue(Runner &R, int work) {
-  if (R.nsys == 1) {
-    R.RA.one = R.mem[0]->sys;
-    if (!R.reuse) R.RA.one.uz = nullptr;
+  R.RA.sys = R.mem[0]->sys;
+  if (!R.reuse) R.RA.sys.uz = nullptr;
+  if (R.RA.sys.skip) {  // a batch of one whose system sits the launch out
+    CK(cudaEventRecord(R.ev_done, R.stream));
+    return OPM_OK;
   }
   R.RA.work = work;
   cudaLaunchConfig_t cfg = {};

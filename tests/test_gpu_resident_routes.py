@@ -110,3 +110,15 @@ def test_legacy_stream_by_name():
             n0 = sv.timing().launches
             assert sv.solve(b)[1] == opm.OPM_OK
             assert (sv.timing().launches - n0 == 1) == resident
+
+
+def test_batch_of_one_that_sits_out():
+    s = synth.config1()
+    b, v = dev(s.x_true), dev(s.vals)
+    with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v) as sv, opm.Batch([sv.h]) as one:
+        want = sv.solve(b)
+        one.launch([None], [None], [None])
+        assert one.wait() == (opm.OPM_OK, [opm.OPM_OK], [0], [0.0])
+        x = torch.empty_like(b)
+        one.launch([v], [b], [x])
+        assert one.wait()[0] == opm.OPM_OK and torch.equal(x, want[0])
