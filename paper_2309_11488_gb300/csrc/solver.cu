@@ -802,8 +802,11 @@ opm_status resident_create(Runner &R, int max_entries) {
   return OPM_OK;
 }
 
-// Enqueues the resident kernel (work: bits of ResidentWork).
-opm_status resident_enqueue(Runner &R, int work) {
+// Enqueues the resident kernel (work: bits of ResidentWork).  On a stream with
+// a part of the device (a green context, a share under MPS) its grid may not
+// fit at once: *fits is false then, and nothing was enqueued.
+opm_status resident_enqueue(Runner &R, int work, bool *fits) {
+  *fits = true;
   R.RA.sys = R.mem[0]->sys;
   if (!R.reuse) R.RA.sys.uz = nullptr;
   if (R.RA.sys.skip) {  // a batch of one whose system sits the launch out
@@ -822,7 +825,13 @@ opm_status resident_enqueue(Runner &R, int work) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   void *args[] = {&R.RA};
-  CK(cudaLaunchKernelExC(&cfg, work == kResApply ? R.res_apply : R.res_kernel, args));
+  const cudaError_t e = cudaLaunchKernelExC(&cfg, work == kResApply ? R.res_apply : R.res_kernel, args);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    cudaGetLastError();
+    *fits = false;
+    return OPM_OK;
+  }
+  CK(e);
   CK(cudaEventRecord(R.ev_done, R.stream));
   return OPM_OK;
 }
@@ -1049,8 +1058,15 @@ opm_status runner_pull_results(Runner &R) {
 
 // Enqueue (no host wait): optional factorisation, then an optional solve.
 opm_status runner_enqueue(Runner &R, bool factor, bool solve) {
-  if (R.resident) return resident_enqueue(R, (factor ? kResFactor : 0) | (solve ? kResSolve : 0));
-  opm_status s = runner_push(R);
+  opm_status s;
+  if (R.resident) {
+    bool fits;
+    s = resident_enqueue(R, (factor ? kResFactor : 0) | (solve ? kResSolve : 0), &fits);
+    if (s != OPM_OK || fits) return s;
+    R.resident = false;  // for good: the launches per phase need no room at once
+    if ((s = build_graphs(R)) != OPM_OK) return s;
+  }
+  s = runner_push(R);
   if (s != OPM_OK) return s;
   if (factor && solve && R.fs_exec) {
     CK(cudaGraphLaunch(R.fs_exec, R.stream));
@@ -2049,8 +2065,10 @@ opm_status opm_ilu_apply(opm_handle h, const double *r, double *z) {
   Runner &R = *h->run;
   // the resident kernel reads r and writes z in the caller's order (no gather
   // and scatter passes): z may take r's place, but not overlap it otherwise
-  if (R.resident && R.resident_alone && (h->sys.b_in == h->sys.x_out || !overlap(h->sys.b_in, h->sys.x_out, h->n))) {
-    if ((s = resident_enqueue(R, kResApply)) != OPM_OK) return s;
+  bool done = R.resident && R.resident_alone &&
+              (h->sys.b_in == h->sys.x_out || !overlap(h->sys.b_in, h->sys.x_out, h->n));
+  if (done && (s = resident_enqueue(R, kResApply, &done)) != OPM_OK) return s;
+  if (done) {
     h->timing.launches += 1;
   } else {
     if ((s = runner_push(R)) != OPM_OK) return s;

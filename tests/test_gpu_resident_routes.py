@@ -1,4 +1,6 @@
 """Which calls go to the resident kernel, and what they report."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -122,3 +124,35 @@ def test_batch_of_one_that_sits_out():
         x = torch.empty_like(b)
         one.launch([v], [b], [x])
         assert one.wait()[0] == opm.OPM_OK and torch.equal(x, want[0])
+
+
+def test_stream_with_a_part_of_the_device():
+    """A green context of 16 SMs cannot hold a quarter of the device's CTAs at once: the launches per phase."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    if not hasattr(cu, "cuGreenCtxStreamCreate"):
+        pytest.skip("this driver has no green contexts")
+    torch.zeros(1, device="cuda")
+    device, whole, part = ctypes.c_int(), ctypes.create_string_buffer(144), ctypes.create_string_buffer(144)
+    groups, desc, ctx, stream = ctypes.c_uint(1), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    assert cu.cuDeviceGet(ctypes.byref(device), 0) == 0
+    assert cu.cuDeviceGetDevResource(device, whole, 1) == 0  # CU_DEV_RESOURCE_TYPE_SM
+    assert cu.cuDevSmResourceSplitByCount(part, ctypes.byref(groups), whole, None, 0, 16) == 0
+    assert cu.cuDevResourceGenerateDesc(ctypes.byref(desc), part, 1) == 0
+    assert cu.cuGreenCtxCreate(ctypes.byref(ctx), desc, device, 1) == 0  # CU_GREEN_CTX_DEFAULT_STREAM
+    assert cu.cuGreenCtxStreamCreate(ctypes.byref(stream), ctx, 1, 0) == 0  # CU_STREAM_NON_BLOCKING
+    try:
+        s = synth.config3(14)
+        b, v = dev(s.x_true), dev(s.vals)
+        torch.cuda.synchronize()
+        out = []
+        for where in (None, stream.value):
+            with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, stream=where) as sv:
+                x, z = torch.empty_like(b), torch.empty_like(b)
+                torch.cuda.synchronize()
+                sv.launch(v, b, x, rtol=1e-6)
+                out.append((sv.wait(), x, sv.ilu_apply(b, z)))
+        assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][2], out[1][2])
+    finally:
+        torch.cuda.synchronize()
+        cu.cuStreamDestroy_v2(stream)
+        cu.cuGreenCtxDestroy(ctx)
