@@ -789,12 +789,13 @@ __global__ void __launch_bounds__(256, 8) k_spmv_v(Batch B) {
 enum TreeMode { kTreeNone = 0, kTreeAll = 1, kTreeMixed = 2 };
 
 // t = A s^, (t,s), (t,t), (s,s); the half-step test and omega.  REUSE as
-// for k_spmv_v.  WIDE: eight CTAs per SM (32 registers; with REUSE its
-// three sums spill 56 bytes per thread), for launches with more tiles than
-// six CTAs per SM hold; otherwise (REUSE) six CTAs per SM and no spill,
-// which a small system's latency-bound product prefers.
+// for k_spmv_v.  WIDE: eight CTAs per SM (32 registers; its three sums spill
+// 56 bytes per thread with REUSE, 48 without), for launches with more tiles
+// than six CTAs per SM hold; otherwise six CTAs per SM and no spill, which a
+// small system's latency-bound product prefers (8 systems, FP32 factors: 420
+// -> 401 us per refactor + solve, 24 systems 630 -> 606).
 template <bool REUSE, bool WIDE, int TREE>
-__global__ void __launch_bounds__(256, (REUSE && !WIDE) ? 6 : 8) k_spmv_t(Batch B) {
+__global__ void __launch_bounds__(256, WIDE ? 8 : 6) k_spmv_t(Batch B) {
   pdl_enter();
   OPM_TILE_S(B, S, lt);
   if (!running(S.st)) return;

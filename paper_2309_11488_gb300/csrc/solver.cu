@@ -431,9 +431,11 @@ int launch_factor_seq(Runner &R, cudaStream_t st) {
 
 template <int TREE>
 void launch_spmv_t(Runner &R, cudaStream_t st) {
-  if (R.reuse && R.ntiles_s > 6 * R.sms) launch_pdl(k_spmv_t<true, true, TREE>, R.ntiles_s, 256, st, R.B);
+  const bool wide = R.ntiles_s > 6 * R.sms;
+  if (R.reuse && wide) launch_pdl(k_spmv_t<true, true, TREE>, R.ntiles_s, 256, st, R.B);
   else if (R.reuse) launch_pdl(k_spmv_t<true, false, TREE>, R.ntiles_s, 256, st, R.B);
-  else launch_pdl(k_spmv_t<false, true, TREE>, R.ntiles_s, 256, st, R.B);
+  else if (wide) launch_pdl(k_spmv_t<false, true, TREE>, R.ntiles_s, 256, st, R.B);
+  else launch_pdl(k_spmv_t<false, false, TREE>, R.ntiles_s, 256, st, R.B);
 }
 
 // One BiCGStab iteration.  With ev (6 events), the kernel groups are
