@@ -156,3 +156,21 @@ def test_stream_with_a_part_of_the_device():
         torch.cuda.synchronize()
         cu.cuStreamDestroy_v2(stream)
         cu.cuGreenCtxDestroy(ctx)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("big", [8, 32, 70])  # rows past the resident kernel's sizes with 70: two orders of summation
+def test_batches_have_the_bits_of_each_alone(big, precision):
+    systems = [synth.config3(big), synth.config1(), synth.chain_system(33)]
+    b, v = [dev(s.x_true) for s in systems], [dev(s.vals) for s in systems]
+    sv = [opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), a, precision=precision) for s, a in zip(systems, v)]
+    alone = [h.solve(c, rtol=1e-4) for h, c in zip(sv, b)]
+    with opm.Batch([h.h for h in sv]) as batch:
+        x = [torch.empty_like(c) for c in b]
+        batch.launch(v, b, x, rtol=1e-4)
+        st, each, iters, relres = batch.wait()
+    assert st == opm.OPM_OK
+    for k, (xa, sa, ia, ra) in enumerate(alone):
+        assert (each[k], iters[k], relres[k]) == (sa, ia, ra) and torch.equal(x[k], xa)
+    for h in sv:
+        h.close()
