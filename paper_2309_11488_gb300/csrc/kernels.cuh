@@ -35,8 +35,9 @@ namespace opm {
 enum SweepMode { kModePlain = 0, kModeP = 1, kModeS = 2 };
 
 // One system's device data.  The last group of fields is set per call.  Not
-// aligned to 16 bytes: the kernels then load neighbouring fields together and
-// wait for both, 0.06 us per launch of a phase of one slice.
+// declared aligned to 16 bytes: the sweeps would load neighbouring fields
+// together and wait for both, 0.06 us per launch of a phase of one slice (the
+// tile kernels prefer it so, see aligned16).
 struct Sys {
   int32_t n, nslices, ntiles, nphases;
   int32_t ntiles_s;  // 256-row tiles of the SpMV kernels
@@ -93,7 +94,9 @@ struct Sys {
   double rtol;
   int32_t maxit;
   int32_t skip;          // the system sits this batch launch out: no kernel touches it
+  int64_t pad3;
 };
+static_assert(sizeof(Sys) % 16 == 0, "the descriptors of an array are aligned to 16 bytes (aligned16)");
 
 // A launchable set of systems (kernel parameter).
 struct Batch {
@@ -665,14 +668,20 @@ __device__ __forceinline__ void row_operator_applied(const Sys &S, const double 
 // t + 768 of the tile); SpMV kernels use tiles of kSpmvRows = 256 rows, one
 // row per thread, so that their last partial wave stays short.
 
-#define OPM_TILE(B, S, lt)                  \
-  const int2 tile_ = (B).tiles[blockIdx.x]; \
-  const Sys &S = (B).sys[tile_.x];          \
+// A descriptor of a launch's array, which is aligned to 16 bytes: its fields
+// are loaded in pairs (949,871 rows, FP64: 3435 -> 3427 us per step).
+__device__ __forceinline__ const Sys &aligned16(const Sys &S) {
+  return *static_cast<const Sys *>(__builtin_assume_aligned(&S, 16));
+}
+
+#define OPM_TILE(B, S, lt)                        \
+  const int2 tile_ = (B).tiles[blockIdx.x];       \
+  const Sys &S = aligned16((B).sys[tile_.x]);     \
   const int lt = tile_.y
 
-#define OPM_TILE_S(B, S, lt)                  \
-  const int2 tile_ = (B).tiles_s[blockIdx.x]; \
-  const Sys &S = (B).sys[tile_.x];            \
+#define OPM_TILE_S(B, S, lt)                      \
+  const int2 tile_ = (B).tiles_s[blockIdx.x];     \
+  const Sys &S = aligned16((B).sys[tile_.x]);     \
   const int lt = tile_.y
 
 #define OPM_TILE_ROWS(i, lt) \
@@ -790,10 +799,11 @@ enum TreeMode { kTreeNone = 0, kTreeAll = 1, kTreeMixed = 2 };
 
 // t = A s^, (t,s), (t,t), (s,s); the half-step test and omega.  REUSE as
 // for k_spmv_v.  WIDE: eight CTAs per SM (32 registers; its three sums spill
-// 56 bytes per thread with REUSE, 48 without), for launches with more tiles
-// than six CTAs per SM hold; otherwise six CTAs per SM and no spill, which a
-// small system's latency-bound product prefers (8 systems, FP32 factors: 420
-// -> 401 us per refactor + solve, 24 systems 630 -> 606).
+// 44 to 64 bytes per thread with REUSE, 48 without where both orders of
+// summation occur), for launches with more tiles than six CTAs per SM hold;
+// otherwise six CTAs per SM and no spill, which a small system's latency-bound
+// product prefers (8 systems, FP32 factors: 420 -> 401 us per refactor +
+// solve, 24 systems 630 -> 606).
 template <bool REUSE, bool WIDE, int TREE>
 __global__ void __launch_bounds__(256, WIDE ? 8 : 6) k_spmv_t(Batch B) {
   pdl_enter();
@@ -934,7 +944,9 @@ __global__ void __launch_bounds__(256, 4) k_update(Batch B) {
 __global__ void __launch_bounds__(256, 8) k_finish(Batch B) {
   __shared__ RedShared<1> rs_;
   red_begin<1>(rs_);
-  OPM_TILE_S(B, S, lt);
+  const int2 tile_ = B.tiles_s[blockIdx.x];
+  const Sys &S = B.sys[tile_.x];  // loaded in pairs, 48 bytes per thread are spilled
+  const int lt = tile_.y;
   if (S.skip) return;
   const int status = S.st->status;
   const bool ok = (status == OPM_OK || status == OPM_NOT_CONVERGED) && S.st->error == 0;
