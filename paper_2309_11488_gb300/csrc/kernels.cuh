@@ -21,9 +21,9 @@
 // 4.4).  The sweeps walk the phases in order, either one launch per phase
 // or one cooperative launch with a bounded grid barrier between phases.
 //
-// Reductions: per system in a fixed order (see red_end); the warp that
-// completes a system's sum runs the scalar part of BiCGStab (alpha, omega,
-// beta, the stopping rule).
+// Reductions: per system in a fixed order (see red_end, last_cta_reduce and
+// last_cta_groups); the warp that completes a system's sum runs the scalar
+// part of BiCGStab (alpha, omega, beta, the stopping rule).
 #pragma once
 
 #include <cstdint>

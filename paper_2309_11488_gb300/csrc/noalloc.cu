@@ -112,9 +112,9 @@ __device__ __forceinline__ void copy8_async(double *dst, const double *src) {
 // the columns and one for the vector at every block) and one thread summed
 // all partials.  A group whose rows are not consecutive (a pattern fault)
 // still reads its blocks in place.
-// Measured, whole call: 2,590 rows 36.9 -> 25.7 us, 249,053 rows 169.8 -> 77.8,
-// 949,871 rows 582.4 -> 199.7 (one group per warp: 115 and 272, the sums'
-// additions costing as much as the product).
+// Measured, whole call: 2,590 rows 37.6 -> 26.8 us, 249,053 rows 173.9 -> 77.3,
+// 949,871 rows 588.9 -> 196.3 (one group per warp: 115 and 272 for the last
+// two, the sums' additions costing as much as the product).
 __global__ void __launch_bounds__(kNaThreads, 8) k_residual_noalloc(
     int32_t nb, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
     const double *__restrict__ vals, const double *__restrict__ x, const double *__restrict__ b,

@@ -4,8 +4,8 @@
 // ILU0 factors and its Krylov vectors.  Work is launched through a Runner: a
 // set of systems (a handle's own set of one, or a batch of handles) with its
 // work lists and its kernel-parameter block.  A single system of the resident
-// kernel's sizes (resident_size) is refactored and solved by one launch of
-// it; everything else goes through three CUDA graphs:
+// kernel's sizes and phases (resident_create) is refactored and solved by one
+// launch of it; everything else goes through three CUDA graphs:
 //   * factor graph: clear errors -> ILU0 phases -> record errors -> results;
 //   * solve graph: setup -> while (any system running) { `chunk` BiCGStab
 //     iterations; loop condition } -> true residual -> results.  The loop
