@@ -110,7 +110,8 @@ struct Runner {
   int iter_launches = 0, factor_launches = 0;
   int tree = kTreeNone;   // which systems' sums take the tree's order (Sys::tree)
   bool resident = false;  // factorisation and solve run in the resident kernel
-  bool resident_alone = false;  // and an application alone does
+  bool resident_solves = false; // so does a solve on kept factors (else it keeps its graph)
+  bool resident_alone = false;  // and an application alone
   Resident RA{};          // its arguments
   const void *res_kernel = nullptr, *res_apply = nullptr;
   int res_grid = 1, res_threads = 256;
@@ -668,10 +669,13 @@ bool resident_size(int nslices, int sms) {
 //            86,518 rows, 22 phases   1285 -> 1899 / 17885 -> 25904; FP32 1182 -> 1462 / 13786 -> 26318
 //            205,187 rows, 250 phases 11782 -> 20837 / 63488 -> 130883
 //   1,218 phases, 120,000 rows (warps) 97497 -> 78925; 2,004 phases, 16,000 rows 126072 -> 55155
+// By trios the factorisation gains at any number of phases and a solve on kept
+// factors up to about 200: past that only calls that refactor are resident.
 bool resident_phases(int nphases, int nslices, bool trio, bool fp32) {
-  if (nphases > kMaxPhaseLaunches) return true;
-  return trio ? nphases <= 192 : nphases <= (fp32 ? 8 : 5) || nslices >= 1000 * (int64_t)nphases;
+  if (nphases > kMaxPhaseLaunches || trio) return true;
+  return nphases <= (fp32 ? 8 : 5) || nslices >= 1000 * (int64_t)nphases;
 }
+bool resident_solve(int nphases, bool trio) { return nphases > kMaxPhaseLaunches || !trio || nphases <= 192; }
 
 // The same for an application alone, which has the phases' stages and nothing
 // else, launches -> resident: trios, FP64, 128 phases 655 -> 638, 299 phases
@@ -747,6 +751,7 @@ opm_status resident_create(Runner &R, int max_entries) {
   if (R.mem[0]->an.max_chain > kResidentChain) return OPM_OK;
   const bool trio = resident_trios(R.nall, R.sms);
   if (!resident_phases(R.nphases, R.nall, trio, R.fp32)) return OPM_OK;
+  R.resident_solves = resident_solve(R.nphases, trio);
   R.resident_alone = resident_apply(R.nphases, R.nall, trio, R.fp32);
   R.res_kernel = R.fp32 ? resident_kernel<float>(trio, false) : resident_kernel<double>(trio, false);
   R.res_apply = R.fp32 ? resident_kernel<float>(trio, true) : resident_kernel<double>(trio, true);
@@ -1011,7 +1016,7 @@ opm_status runner_create(const std::vector<opm_solver *> &mem, cudaStream_t stre
       }
   }
   if (sweep_launch == OPM_SWEEP_AUTO && !profile && (s = resident_create(*R, max_entries)) != OPM_OK) return fail(s);
-  if (!R->resident && (s = build_graphs(*R)) != OPM_OK) return fail(s);
+  if (!(R->resident && R->resident_solves) && (s = build_graphs(*R)) != OPM_OK) return fail(s);
   if (cudaStreamSynchronize(stream) != cudaSuccess) {
     cudaGetLastError();
     return fail(OPM_ERR_CUDA);
@@ -1027,7 +1032,7 @@ opm_status runner_sync_wells(Runner &R) {
   bool any = false;
   for (auto *h : R.mem) any = any || h->sys.nwells > 0;
   if (any == R.has_wells) return OPM_OK;
-  if (R.resident) {  // no graphs: the kernel looks at the wells itself
+  if (!R.solve_exec) {  // no graphs: the resident kernel looks at the wells itself
     R.has_wells = any;
     return OPM_OK;
   }
@@ -1058,15 +1063,18 @@ opm_status runner_pull_results(Runner &R) {
   return OPM_OK;
 }
 
+// Whether a call goes to the resident kernel.
+bool resident_call(const Runner &R, bool factor) { return R.resident && (factor || R.resident_solves); }
+
 // Enqueue (no host wait): optional factorisation, then an optional solve.
 opm_status runner_enqueue(Runner &R, bool factor, bool solve) {
   opm_status s;
-  if (R.resident) {
+  if (resident_call(R, factor)) {
     bool fits;
     s = resident_enqueue(R, (factor ? kResFactor : 0) | (solve ? kResSolve : 0), &fits);
     if (s != OPM_OK || fits) return s;
     R.resident = false;  // for good: the launches per phase need no room at once
-    if ((s = build_graphs(R)) != OPM_OK) return s;
+    if (!R.solve_exec && (s = build_graphs(R)) != OPM_OK) return s;
   }
   s = runner_push(R);
   if (s != OPM_OK) return s;
@@ -1086,9 +1094,10 @@ opm_status runner_wait(Runner &R) {
   return OPM_OK;
 }
 
-// Kernel launches of one solve-graph execution, for the launch counter.
-int64_t solve_graph_launches(const Runner &R) {
-  if (R.resident) return 1;
+// Kernel launches of one solve (with the factorisation, if resident), for the
+// launch counter.
+int64_t solve_launches(const Runner &R, bool factor) {
+  if (resident_call(R, factor)) return 1;
   int maxit = 1;
   for (int s = 0; s < R.nsys; ++s) maxit = std::max(maxit, R.h_res[s].iters);
   const int64_t bodies = (maxit + R.chunk - 1) / R.chunk;
@@ -1956,7 +1965,7 @@ opm_status opm_bicgstab_solve(opm_handle h, const double *b, double *x, double r
   } else {
     if ((s = runner_enqueue(R, false, true)) != OPM_OK) return s;
     if ((s = runner_wait(R)) != OPM_OK) return s;
-    h->timing.launches += solve_graph_launches(R);
+    h->timing.launches += solve_launches(R, false);
   }
   if (!x_dev) CK(cudaMemcpyAsync(x, h->vec_out, vbytes, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaEventRecord(h->ev[1], h->stream));
@@ -1990,7 +1999,7 @@ opm_status opm_solve_launch(opm_handle h, const double *vals, const double *b, d
   }
   h->async_pending = true;
   h->async_factor = vals != nullptr;
-  h->timing.launches += vals ? h->run->factor_launches : 0;
+  h->timing.launches += vals && !R.resident ? R.factor_launches : 0;
   return OPM_OK;
 }
 
@@ -2009,7 +2018,7 @@ opm_status opm_solve_wait(opm_handle h, int32_t *iters, double *relres) {
   opm_status s = runner_wait(R);
   if (s != OPM_OK) return s;
   const Result &r = R.h_res[0];
-  h->timing.launches += solve_graph_launches(R);
+  h->timing.launches += solve_launches(R, h->async_factor);
   if (r.status == OPM_ERR_ZERO_PIVOT) {
     h->factors_ok = false;
     h->last_err_row = (r.err_row >= 0 && r.err_row < h->n) ? h->an.perm[r.err_row] : -1;

@@ -28,38 +28,57 @@ def test_launches_are_counted():
         assert seen == [1, 2, 3, 4, 5]
 
 
-# (system, schedule, partitions, precision): whether the resident kernel solves it, and applies it alone; by phases
+def flat(nx, ny):
+    return synth.grid_system(nx, ny, 1, np.random.default_rng(1).normal(size=(1, ny, nx)), seed=3)
+
+
+# (system, schedule, partitions, precision): whether the resident kernel refactors and solves it, solves it on kept
+# factors, and applies it alone; by phases
 ROUTES = [
-    (lambda: synth.config3(14), "level", 0, "fp64", True, True),  # 47 phases, trios
-    (lambda: synth.config3(14), "level", 0, "fp32", True, False),
-    (lambda: synth.config3(14), "auto", 0, "fp32", True, True),
-    (lambda: synth.chain_system(300), "natural", 0, "fp64", False, False),  # 300 phases
-    (lambda: synth.chain_system(1025), "natural", 0, "fp32", True, True),  # more than launches are made for
-    (lambda: synth.config3(45), "auto", 0, "fp64", True, True),  # 3 phases, a warp per slice
-    (lambda: synth.config3(45), "level", 512, "fp64", False, False),  # 22 phases
+    (lambda: synth.config3(14), "level", 0, "fp64", True, True, True),  # 47 phases, trios
+    (lambda: synth.config3(14), "level", 0, "fp32", True, True, False),
+    (lambda: synth.config3(14), "auto", 0, "fp32", True, True, True),
+    (lambda: synth.chain_system(192), "natural", 0, "fp64", True, True, True),
+    (lambda: synth.chain_system(193), "natural", 0, "fp64", True, False, False),
+    (lambda: flat(200, 15), "level", 0, "fp32", True, False, False),  # 214 phases
+    (lambda: synth.chain_system(1025), "natural", 0, "fp32", True, True, True),  # more than launches are made for
+    (lambda: synth.config3(45), "auto", 0, "fp64", True, True, True),  # 3 phases, a warp per slice
+    (lambda: synth.config3(45), "level", 512, "fp64", False, False, False),  # 22 phases
 ]
 
 
-@pytest.mark.parametrize("make, schedule, parts, precision, solves, applies", ROUTES)
-def test_routes_by_phases(make, schedule, parts, precision, solves, applies):
-    """A route is seen in the kernels that a call launches; the bits are those of the launches per phase."""
+@pytest.mark.parametrize("make, schedule, parts, precision, steps, solves, applies", ROUTES)
+@pytest.mark.parametrize("nwells", [0, 2])
+def test_routes_by_phases(make, schedule, parts, precision, steps, solves, applies, nwells):
+    """A route is seen in the kernels that a call launches; the bits are those of the launches per phase, also when
+    wells come and go between calls."""
     s = make()
     part = np.ascontiguousarray(synth.partition_grid(s, parts), dtype=np.int32) if parts else None
+    if nwells and s.nb < 2000:
+        pytest.skip("wells are placed on grids")
     b, v = dev(s.x_true), dev(s.vals)
     out = []
     for sweep in ("per_phase", "auto"):
         with opm.Solver(s.nb, dev(s.rowptr), dev(s.colidx), v, schedule=schedule, precision=precision, part=part,
                         sweep_launch=sweep) as sv:
             x = torch.empty_like(b)
-            n0 = sv.timing().launches
+            got, n = [], [sv.timing().launches]
+            if nwells:
+                assert sv.set_wells(synth.wells(s, nwells, 4)) == opm.OPM_OK
             sv.launch(v, b, x, rtol=1e-4)
-            got = sv.wait()
-            n1 = sv.timing().launches
-            z = sv.ilu_apply(b)
-            n2 = sv.timing().launches
-            out.append((got, x, z))
-    assert (n1 - n0 == 1) == solves and (n2 - n1 == 1) == applies
-    assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1]) and torch.equal(out[0][2], out[1][2])
+            got += [sv.wait(), x]
+            n.append(sv.timing().launches)
+            got += sv.solve(b, rtol=1e-4)
+            n.append(sv.timing().launches)
+            got.append(sv.ilu_apply(b))
+            n.append(sv.timing().launches)
+            if nwells:
+                assert sv.set_wells(None) == opm.OPM_OK
+                got += sv.solve(b, rtol=1e-4)
+            out.append(got)
+    assert [k == 1 for k in np.diff(n)] == [steps, solves, applies]
+    for p, q in zip(*out):
+        assert torch.equal(p, q) if torch.is_tensor(p) else p == q
 
 
 def test_edges_of_the_three_warp_form():
@@ -67,11 +86,10 @@ def test_edges_of_the_three_warp_form():
     44,431-row mesh.  The limit follows from the number of SMs."""
     slices = 5 * 5 * torch.cuda.get_device_properties(0).multi_processor_count // 2
     side = round((32 * slices) ** 0.5 / 8) * 8
-    logk = lambda *d: np.random.default_rng(1).normal(size=d)
     systems = [synth.config2()]
     for rows in (32 * slices, 32 * slices + 1):  # chains: any row count
         systems.append(synth.chain_system(rows))
-    systems.append(synth.grid_system(side, 32 * slices // side, 1, logk(1, 32 * slices // side, side), seed=3))
+    systems.append(flat(side, 32 * slices // side))
     for s in systems:
         for precision in ("fp64", "fp32"):
             b, v = dev(s.x_true), dev(s.vals)
